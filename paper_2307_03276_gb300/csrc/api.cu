@@ -190,7 +190,8 @@ static int next_pow2(int v) {
 // for the blocks per SM the tile kernel is built for (four with one float4 per
 // lane, else three).  With materialised Khatri-Rao rows the stage holds only
 // row ids and values, so the same room takes larger tiles.
-static void heuristic_config(const cpapr_ctx *ctx, int n, int pi, int *lanes, int *tile, int *reduction) {
+static void heuristic_config(const cpapr_ctx *ctx, int n, int pi, int *lanes, int *tile, int *reduction,
+                             int *batch_sh) {
     const int Rp = ctx->Rp;
     int g;
     if (ctx->esize == 8)
@@ -210,6 +211,24 @@ static void heuristic_config(const cpapr_ctx *ctx, int n, int pi, int *lanes, in
                 break;
             }
     }
+    // A tensor that would give only a few tiles takes smaller ones instead: its
+    // launch lasts as long as one tile's serial walk, so the walk is shortened
+    // until the tiles fill the SMs.  FP64: the smallest power of two from 64 on
+    // with fewer than 4 tiles per SM, within 5% of the best of {64, .., 2048} for
+    // 3e3 to 1e6 nonzeros at R = 8, 16, 32 (an inner iteration of 1e4 nonzeros,
+    // R = 16: 149 us at 2048 nonzeros per tile, 33 at 64; 1e5: 96 -> 41; 3e5:
+    // 79 -> 56); beyond it the rows cut by more tiles cost more than the shorter
+    // walk saves (1e5 at 64: 51 us, 1e6: 290).  The batched solver, whose launch
+    // holds the tiles of many tensors, keeps the large ones (64 tensors 80 ms, 91
+    // in these small ones).  FP32, whose walks are shorter: the smallest from 256
+    // on with at most one tile per SM (1e4 37 -> 24 us, 1e5 34 -> 28), which the
+    // batched solver takes too, so that a tensor's sums keep one order in both.
+    *batch_sh = 0;
+    const bool f64 = ctx->esize == 8;
+    while (*tile > (f64 ? 64 : 256) && ceil_div(ctx->nnz, *tile / 2) < (f64 ? kSmallTiles : kSmallTiles / 4)) {
+        *tile /= 2;
+        *batch_sh += f64 ? 1 : 0;
+    }
     *reduction = CPAPR_REDUCE_SEGMENTED;
     (void)n;
 }
@@ -225,6 +244,7 @@ cpapr_status configure_mode(cpapr_ctx *ctx, int n, int lanes, int tile, int redu
     if (phi_smem_for((int)ctx->esize, ctx->N - 1, tile, ctx->Rp, lanes) > kMaxPhiSmem)
         return fail(ctx, CPAPR_E_ARG, "tile_nnz too large: its staged streams and partial rows exceed shared memory");
     ModeLayout &L = ctx->mode[n];
+    L.batch_sh = 0;
     L.lanes = lanes;
     L.reduction = reduction == CPAPR_REDUCE_ATOMIC ? CPAPR_REDUCE_ATOMIC : CPAPR_REDUCE_SEGMENTED;
     if (L.tile_nnz != tile || !L.row_first) CPAPR_TRY(build_tiles(ctx, n, tile));
@@ -492,13 +512,14 @@ cpapr_status cpapr_create(int32_t nmodes, const int64_t *dims, int64_t nnz, cons
     if (o.l2_persist) CR_TRY(configure_l2_window(ctx));
 
     for (int n = 0; n < nmodes; ++n) {
-        int lanes, tile, red;
+        int lanes, tile, red, batch_sh;
         const int pi = o.pi_mode == CPAPR_PI_MATERIALISED ? 1 : o.pi_mode == CPAPR_PI_FUSED ? 0 : pi_auto(ctx);
-        heuristic_config(ctx, n, pi, &lanes, &tile, &red);
+        heuristic_config(ctx, n, pi, &lanes, &tile, &red, &batch_sh);
         if (o.rank_lanes) lanes = o.rank_lanes;
         if (o.tile_nnz) tile = o.tile_nnz;
         if (o.reduction) red = o.reduction;
         CR_TRY(configure_mode(ctx, n, lanes, tile, red));
+        if (!o.tile_nnz) ctx->mode[n].batch_sh = batch_sh;
         CR_TRY(configure_pi(ctx, n, pi));
     }
     if (o.autotune || o.tune_cache) CR_TRY(autotune(ctx));

@@ -600,11 +600,15 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
         const int lanes = Classes<T>::g[k];
         for (int n = 0; n < N; ++n) {
             ModeLayout &L = ctxs[i]->mode[n];
-            int tile = L.tile_nnz;
-            while (tile > 256 && phi_smem_bytes(tile, N - 1, (int)sizeof(T), batch_threads<T>(), maxrpl) > budget)
-                tile /= 2;
+            int tile = L.tile_nnz, sh = L.batch_sh;
+            auto over = [&](int t) {
+                return phi_smem_bytes(t, N - 1, (int)sizeof(T), batch_threads<T>(), maxrpl) > budget;
+            };
+            while (sh > 0 && over(tile << sh)) --sh;
+            while (tile > 256 && over(tile)) tile /= 2;
             if (L.lanes != lanes || L.reduction != CPAPR_REDUCE_SEGMENTED || tile != L.tile_nnz)
                 CPAPR_TRY(configure_mode(ctxs[i], n, lanes, tile, CPAPR_REDUCE_SEGMENTED));
+            L.batch_sh = sh;
         }
         CPAPR_CUDA(ctxs[i], cudaStreamSynchronize(ctxs[i]->stream));
     }
@@ -677,8 +681,10 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
             std::memset(&d, 0, sizeof(d));
             PhiArgs &a = d.a;
             a.nnz = c->nnz;
-            a.T = L.tile_nnz;
-            a.ntiles = L.ntiles;
+            a.T = L.tile_nnz << L.batch_sh;
+            a.ntiles = (int32_t)ceil_div(c->nnz, a.T);
+            a.ksh = L.batch_sh;
+            a.ntab = L.ntiles;
             a.Rp = c->Rp;
             a.In = L.In;
             a.nm1 = c->N - 1;
@@ -729,7 +735,7 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
             d.kappa_tol = c->opt.kappa_tol;
             d.erows = L.erows;
             d.nempty = c->nnz > 0 ? L.nempty : 0;
-            for (int t = 0; t < (c->nnz > 0 ? L.ntiles : 0); ++t) tiles.push_back(make_int2(i, t));
+            for (int t = 0; t < (c->nnz > 0 ? a.ntiles : 0); ++t) tiles.push_back(make_int2(i, t));
             for (int t = 0; t < d.nchunks; ++t) chunks.push_back(make_int2(i, t));
             for (int t = 0; t < (int)ceil_div(d.nempty * c->Rp, kEmptyChunk); ++t) echunks.push_back(make_int2(i, t));
         }
@@ -740,7 +746,7 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
         mp.ntiles = (int)tiles.size();
         {
             int maxtile = 4;
-            for (int i = 0; i < count; ++i) maxtile = std::max(maxtile, ctxs[i]->mode[n].tile_nnz);
+            for (int i = 0; i < count; ++i) maxtile = std::max(maxtile, desc[i].a.T);
             mp.smem = phi_smem_bytes(maxtile, N - 1, (int)sizeof(T), batch_threads<T>(), maxrpl);
             smem_max = std::max(smem_max, mp.smem);
         }
@@ -768,7 +774,7 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
         for (int i = 0; i < count; ++i) {
             desc0[i].a.inner = nullptr;
             desc0[i].a.pi = nullptr;
-            const int nll = ctxs[i]->nnz > 0 ? ctxs[i]->mode[0].ntiles : 0;
+            const int nll = ctxs[i]->nnz > 0 ? desc0[i].a.ntiles : 0;
             args[i] = ll_total_args(ctxs[i], ctxs[i]->llpart, nll, P.ll + i);
             for (int b = 0; b < args[i].part0[N]; ++b) items.push_back(make_int2(i, b));
         }

@@ -20,8 +20,8 @@
 //   4. gather the other modes' coordinates and the values in sorted order;
 //   5. tile tables: tiles of tile_nnz consecutive sorted nonzeros, the row
 //      holding each tile's first nonzero, the rows that span more than one
-//      tile with, per tile, the split its head and tail partials belong to,
-//      and one counter per split.
+//      tile with, per tile, the split its head partial belongs to, and one
+//      counter per split.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -623,22 +623,20 @@ __global__ void split_write_kernel(const int32_t *__restrict__ seg, const int32_
     }
 }
 
-// tsplit[2t] = split whose row holds tile t's head partial (the row began in
-// an earlier tile), tsplit[2t+1] = split whose first tile is t (tile t's tail
-// partial); -1 where there is none.  pos = exclusive scan of the split-start
+// tsplit[t] = split whose row holds tile t's head partial (the row began in
+// an earlier tile), or -1; tile t's tail partial, of a row that goes on in tile
+// t + 1, belongs to tsplit[t + 1].  pos = exclusive scan of the split-start
 // flags, total = their sum: the splits started at or before tile u number
-// incl(u) = pos[u + 1] (total for the last tile).
+// incl(u) = pos[u + 1] (total for the last tile).  The tables serve tiles of
+// 2^k table tiles as they are: such a tile t begins with table tile t 2^k, and
+// a split's first and last tile are shifted right by k.
 __global__ void tile_split_kernel(const int32_t *__restrict__ seg, const int32_t *__restrict__ row_first, int32_t T,
                                   int32_t ntiles, const uint32_t *__restrict__ pos, const uint32_t *__restrict__ total,
                                   int32_t *__restrict__ tsplit) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= ntiles) return;
     auto incl = [&](int u) -> int32_t { return (int32_t)(u + 1 < ntiles ? pos[u + 1] : *total); };
-    int32_t head = -1, tail = -1;
-    if (t >= 1 && (int64_t)seg[row_first[t]] < (int64_t)t * T) head = incl(t) - 1;
-    if (t + 1 < ntiles && incl(t + 1) - (int32_t)pos[t + 1] == 1) tail = (int32_t)pos[t + 1];
-    tsplit[2 * t] = head;
-    tsplit[2 * t + 1] = tail;
+    tsplit[t] = (t >= 1 && (int64_t)seg[row_first[t]] < (int64_t)t * T) ? incl(t) - 1 : -1;
 }
 
 cpapr_status build_tiles(cpapr_ctx *ctx, int n, int tile_nnz) {
@@ -678,7 +676,7 @@ cpapr_status build_tiles(cpapr_ctx *ctx, int n, int tile_nnz) {
         CPAPR_CUDA(ctx, lib_malloc((void **)&L.split, (size_t)std::max<int>(L.nsplit, 1) * 12, s));
         split_write_kernel<<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(L.seg, L.row_first, tile_nnz, nt, flag, L.split);
         CPAPR_CUDA(ctx, cudaGetLastError());
-        CPAPR_CUDA(ctx, lib_malloc((void **)&L.tsplit, (size_t)nt * 8, s));
+        CPAPR_CUDA(ctx, lib_malloc((void **)&L.tsplit, (size_t)nt * 4, s));
         tile_split_kernel<<<(unsigned)ceil_div(nt, 256), 256, 0, s>>>(L.seg, L.row_first, tile_nnz, nt, flag, dtot,
                                                                       L.tsplit);
         count_launch(ctx);
@@ -686,8 +684,8 @@ cpapr_status build_tiles(cpapr_ctx *ctx, int n, int tile_nnz) {
         CPAPR_CUDA(ctx, cudaFreeAsync(flag, s));
     } else {
         CPAPR_CUDA(ctx, lib_malloc((void **)&L.split, 12, s));
-        CPAPR_CUDA(ctx, lib_malloc((void **)&L.tsplit, (size_t)std::max(nt, 1) * 8, s));
-        CPAPR_CUDA(ctx, cudaMemsetAsync(L.tsplit, 0xff, (size_t)std::max(nt, 1) * 8, s));
+        CPAPR_CUDA(ctx, lib_malloc((void **)&L.tsplit, (size_t)std::max(nt, 1) * 4, s));
+        CPAPR_CUDA(ctx, cudaMemsetAsync(L.tsplit, 0xff, (size_t)std::max(nt, 1) * 4, s));
     }
     CPAPR_CUDA(ctx, lib_malloc((void **)&L.splitcnt, (size_t)std::max(L.nsplit, 1) * 4, s));
     CPAPR_CUDA(ctx, cudaMemsetAsync(L.splitcnt, 0, (size_t)std::max(L.nsplit, 1) * 4, s));

@@ -61,8 +61,9 @@ struct ModeLayout {
     int32_t *krow = nullptr;       // [ntiles + 1] index in nzrow of that row; krow[ntiles] = K - 1
     int32_t nsplit = 0;
     int32_t *split = nullptr;      // [3 * nsplit] (row, first tile, last tile)
-    int32_t *tsplit = nullptr;     // [2 * ntiles] split of each tile's head / tail partial, or -1
+    int32_t *tsplit = nullptr;     // [ntiles] split of each tile's head partial, or -1
     int32_t *splitcnt = nullptr;   // [nsplit] partial counters of the tile kernel (zero between launches)
+    int32_t batch_sh = 0;          // the batched solver takes 2^batch_sh of these tiles as one (heuristic_config)
     int32_t pi = 0;                // 1: Phi streams the materialised Khatri-Rao rows (built per outer iteration)
     int32_t nempty = 0;
     int32_t *erows = nullptr;      // [nempty] rows without nonzeros, increasing
@@ -139,6 +140,8 @@ namespace cpapr {
 constexpr int kColParts = 256;
 // tiles from which an FP64 Phi launch takes the kernel with its dot on the FP32 pipe
 constexpr int kDfMinTiles = 152 * 4;
+// below this many tiles the automatic tile size shrinks (heuristic_config)
+constexpr int kSmallTiles = 152 * 4;
 
 // ---- error plumbing ------------------------------------------------------
 cpapr_status fail(cpapr_ctx *ctx, cpapr_status st, const std::string &msg);

@@ -77,6 +77,8 @@ static PhiArgs make_args(cpapr_ctx *ctx, int n, const void *B, void *out, InnerS
     a.nnz = ctx->nnz;
     a.T = L.tile_nnz;
     a.ntiles = L.ntiles;
+    a.ksh = 0;
+    a.ntab = L.ntiles;
     a.Rp = ctx->Rp;
     a.In = L.In;
     a.nm1 = ctx->N - 1;

@@ -57,21 +57,23 @@ struct PhiArgs {
     int64_t nnz;
     int32_t T;       // nonzeros per tile
     int32_t ntiles;
+    int32_t ksh;     // log2 of the tables' tiles per tile: T and ntiles count tiles of 2^ksh table tiles
+    int32_t ntab;    // tiles of the tables (krow, tsplit, split)
     int32_t Rp;
     int32_t In;
     int32_t nm1;     // number of gathered modes (N - 1)
     int32_t atomic;  // 1: partial rows are added with atomics into a zeroed output
     const uint32_t *rstart;  // row-start bits of the sorted positions: bit p set where a row begins at p
     const int32_t *nzrow;    // the rows holding nonzeros, increasing
-    const int32_t *krow;     // [ntiles + 1] index in nzrow of the row holding each tile's first nonzero
+    const int32_t *krow;     // [ntab + 1] index in nzrow of the row holding each table tile's first nonzero
     const int32_t *idx[kMaxNm1];
     const void *val;
     const void *A[kMaxNm1];
     const void *B;
     void *out;
     void *carry;     // head partials [ntiles][Rp], then tail partials [ntiles][Rp]
-    const int32_t *split;   // [nsplit][3]: rows that span tiles (row, first tile, last tile)
-    const int32_t *tsplit;  // [ntiles][2]: split of the tile's head partial, of its tail partial (-1: none)
+    const int32_t *split;   // [nsplit][3]: rows that span table tiles (row, first tile, last tile)
+    const int32_t *tsplit;  // [ntab]: split of each table tile's head partial (-1: none)
     int32_t *splitcnt;      // [nsplit]: partials arrived in this launch (zero between launches)
     int32_t nsplit;
     double eps;
@@ -671,8 +673,8 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
     unsigned long long kslot0 = 0ull, kslot1 = 0ull;
     int32_t kl = 0;
     if (threadIdx.x == 0) {
-        k0 = __ldg(a.krow + t);
-        k1 = __ldg(a.krow + t + 1);
+        k0 = __ldg(a.krow + ((int64_t)t << a.ksh));
+        k1 = __ldg(a.krow + min((int64_t)(t + 1) << a.ksh, (int64_t)a.ntab));
         if (KSEED && a.inner) {
             kl = *((volatile int32_t *)&a.inner->l);
             kslot0 = *((volatile unsigned long long *)&a.inner->kkt[0]);
@@ -1205,9 +1207,13 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
                 __threadfence();
                 __syncwarp();
                 if (wlane == 0) {
-                    const int32_t si = __ldg(a.tsplit + 2 * t + (s == 0 ? 0 : 1));
+                    // the row's split: the one of this tile's head partial, or (a row
+                    // that goes on after the tile) of the next tile's
+                    const int64_t ht = (int64_t)(s == 0 ? t : t + 1) << a.ksh;
+                    const int32_t si = ht < a.ntab ? __ldg(a.tsplit + ht) : -1;
                     if (si >= 0 && si < a.nsplit) {  // always, by construction of the table
-                        const int32_t parts = __ldg(a.split + 3 * si + 2) - __ldg(a.split + 3 * si + 1) + 1;
+                        const int32_t parts =
+                            (__ldg(a.split + 3 * si + 2) >> a.ksh) - (__ldg(a.split + 3 * si + 1) >> a.ksh) + 1;
                         if (atomicAdd(a.splitcnt + si, 1) == parts - 1) slot_fin[s == 0 ? 0 : 1] = si;
                     }
                 }
@@ -1225,8 +1231,8 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
             if (si < 0) continue;
             __threadfence();
             const int32_t crow = __ldg(a.split + 3 * si + 0);
-            const int32_t t0 = __ldg(a.split + 3 * si + 1);
-            const int npart = __ldg(a.split + 3 * si + 2) - t0 + 1;
+            const int32_t t0 = __ldg(a.split + 3 * si + 1) >> a.ksh;
+            const int npart = (__ldg(a.split + 3 * si + 2) >> a.ksh) - t0 + 1;
             auto part = [&](int k, int c) -> T {
                 const int64_t off = k == 0 ? ((int64_t)a.ntiles + t0) * Rp : (int64_t)(t0 + k) * Rp;
                 return __ldcg(carry + off + c);
