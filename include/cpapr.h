@@ -85,17 +85,20 @@ enum { CPAPR_DOT_AUTO = 0, CPAPR_DOT_FP64 = 1, CPAPR_DOT_FP32_PIPE = 2 };
  *             its KKT reduction, and for atomic adds the zeroing and the
  *             separate KKT pass they need).  Timing replaces the model; set
  *             one after cpapr_create.
- *  fp64_dot   how the FP64 form's Phi evaluates the divisor's dot product
- *             <B[i_n], pi>.  CPAPR_DOT_FP64: FP64 FMAs.  CPAPR_DOT_FP32_PIPE:
- *             on the FP32 pipe (64 times the FP64 FMA rate on GB300) with
- *             error-free transformations of 48-bit hi/lo cuts of the FP64
- *             operands; its error stays below 6e-13 relative to
- *             max(s, eps), inside the FP64 form's 1e-12 bound (it applies to
- *             lanes of 8 or fewer ranks and eps >= 2^-43; operands >= 2^31 take
- *             the FP64 dot for their batch).  CPAPR_DOT_AUTO (default): the FP32
- *             pipe where a launch has at least 608 tiles (4 per SM), the FP64
- *             dot below that, where one tile's latency bounds the launch.  The
- *             batched solver always takes the FP64 dot.  Ignored in FP32.
+ *  fp64_dot   how the FP64 form evaluates Phi.  CPAPR_DOT_FP64: FP64 FMAs.
+ *             CPAPR_DOT_FP32_PIPE: on the FP32 pipe (64 times the FP64 FMA rate
+ *             on GB300), with the Khatri-Rao rows as pairs of floats (48 and
+ *             more bits; values beyond a pair's range stay FP64) and error-free
+ *             transformations for the dot product, the division and the
+ *             scaled addition; Phi's error stays below 1e-12 relative per entry
+ *             (measured near 1e-14).  It applies where rank_lanes leaves 8 or
+ *             fewer ranks per lane and 2^-43 <= eps <= 2^20; a nonzero outside
+ *             its ranges (a value outside {0} and [2^-20, 2^31), ...) is
+ *             evaluated in FP64.  CPAPR_DOT_AUTO (default): the FP32 pipe where
+ *             the tensor has at least 608 tiles (4 per SM; of 2048 nonzeros, 1024
+ *             from rank 17 on, or of tile_nnz), FP64 below that, where one tile's
+ *             latency bounds the launch.  The batched solver always takes
+ *             FP64.  Ignored in FP32.
  *  tune_cache NULL (default) or the path of a text file of tuned choices,
  *             one line per shape class: precision, number of modes, padded
  *             rank, and power-of-two buckets of the nonzeros, of the mode's
@@ -314,11 +317,11 @@ typedef struct {
     int32_t precision;
     int64_t nnz;
     int64_t dims[CPAPR_MAX_MODES];
-    int32_t tile_nnz[CPAPR_MAX_MODES];    /* chosen per mode */
+    int32_t tile_nnz[CPAPR_MAX_MODES];    /* chosen per mode (of its Phi launches) */
     int32_t rank_lanes[CPAPR_MAX_MODES];  /* chosen per mode */
     int32_t reduction[CPAPR_MAX_MODES];   /* chosen per mode */
     int32_t ntiles[CPAPR_MAX_MODES];
-    int32_t nsplit[CPAPR_MAX_MODES];      /* rows that span more than one tile */
+    int32_t nsplit[CPAPR_MAX_MODES];      /* rows that span tiles (of the smallest tile any launch of the mode takes) */
     int32_t pi_mode[CPAPR_MAX_MODES];     /* CPAPR_PI_FUSED or CPAPR_PI_MATERIALISED, per mode */
     int64_t device_bytes;  /* device memory held by the context */
     int64_t kernel_launches; /* kernels this context has launched (graph replays counted per kernel) */

@@ -190,8 +190,7 @@ static int next_pow2(int v) {
 // for the blocks per SM the tile kernel is built for (four with one float4 per
 // lane, else three).  With materialised Khatri-Rao rows the stage holds only
 // row ids and values, so the same room takes larger tiles.
-static void heuristic_config(const cpapr_ctx *ctx, int n, int pi, int *lanes, int *tile, int *reduction,
-                             int *batch_sh) {
+static void heuristic_config(const cpapr_ctx *ctx, int pi, ModeLayout &L, int *lanes, int *tile, int *reduction) {
     const int Rp = ctx->Rp;
     int g;
     if (ctx->esize == 8)
@@ -220,17 +219,32 @@ static void heuristic_config(const cpapr_ctx *ctx, int n, int pi, int *lanes, in
     // 79 -> 56); beyond it the rows cut by more tiles cost more than the shorter
     // walk saves (1e5 at 64: 51 us, 1e6: 290).  The batched solver, whose launch
     // holds the tiles of many tensors, keeps the large ones (64 tensors 80 ms, 91
-    // in these small ones).  FP32, whose walks are shorter: the smallest from 256
-    // on with at most one tile per SM (1e4 37 -> 24 us, 1e5 34 -> 28), which the
-    // batched solver takes too, so that a tensor's sums keep one order in both.
-    *batch_sh = 0;
+    // in these small ones).
+    // FP32 keeps one tile size whatever the tensor's: its sums keep their order.
     const bool f64 = ctx->esize == 8;
-    while (*tile > (f64 ? 64 : 256) && ceil_div(ctx->nnz, *tile / 2) < (f64 ? kSmallTiles : kSmallTiles / 4)) {
+    const int full = *tile;
+    L.sh = L.sh_df = L.batch_sh = 0;
+    if (f64 && ceil_div(ctx->nnz, full) >= kDfMinTiles) {
+        // Large FP64 launches run on float pairs: tables of small tiles, of which
+        // those launches take as many as leave 9 tiles per SM, up to 128 nonzeros
+        // per group (3-way Zipf, Phi in us at 512 / 1024 / 2048 / 4096 nonzeros per
+        // tile: 7e5 nonzeros, R = 16, 71 / 74 / 93 / 135; 3e6, R = 16, 177 / 146 / 137 /
+        // 137; 6e6, R = 32, 407 / 360 / 343 / 350; 4-way 5e7, R = 16, - / 1836 / 1516 /
+        // 1353, 1315 at 8192); the others, and the batched solver, as many as make
+        // the tile chosen above.
+        *tile = kDfTile;
+        while ((*tile << L.sh) < full) ++L.sh;
+        L.batch_sh = L.sh;
+        const int groups = 128 / std::max(1, Rp / 4);
+        while ((*tile << (L.sh_df + 1)) <= kDfRun * groups &&
+               ceil_div(ctx->nnz, (int64_t)*tile << (L.sh_df + 1)) >= kDfLaunchTiles)
+            ++L.sh_df;
+    }
+    while (f64 && *tile > 64 && ceil_div(ctx->nnz, *tile / 2) < kSmallTiles) {
         *tile /= 2;
-        *batch_sh += f64 ? 1 : 0;
+        ++L.batch_sh;
     }
     *reduction = CPAPR_REDUCE_SEGMENTED;
-    (void)n;
 }
 
 void batch_forget(cpapr_ctx *ctx);
@@ -244,7 +258,7 @@ cpapr_status configure_mode(cpapr_ctx *ctx, int n, int lanes, int tile, int redu
     if (phi_smem_for((int)ctx->esize, ctx->N - 1, tile, ctx->Rp, lanes) > kMaxPhiSmem)
         return fail(ctx, CPAPR_E_ARG, "tile_nnz too large: its staged streams and partial rows exceed shared memory");
     ModeLayout &L = ctx->mode[n];
-    L.batch_sh = 0;
+    L.sh = L.sh_df = L.batch_sh = 0;
     L.lanes = lanes;
     L.reduction = reduction == CPAPR_REDUCE_ATOMIC ? CPAPR_REDUCE_ATOMIC : CPAPR_REDUCE_SEGMENTED;
     if (L.tile_nnz != tile || !L.row_first) CPAPR_TRY(build_tiles(ctx, n, tile));
@@ -260,7 +274,7 @@ cpapr_status configure_mode(cpapr_ctx *ctx, int n, int lanes, int tile, int redu
         cudaGraphExecDestroy(ctx->graph_exec[n]);
         ctx->graph_exec[n] = nullptr;
     }
-    return CPAPR_OK;
+    return ensure_pair_storage(ctx);
 }
 
 // Materialised Khatri-Rao rows: one buffer of nnz_pad x Rp elements shared by
@@ -512,14 +526,20 @@ cpapr_status cpapr_create(int32_t nmodes, const int64_t *dims, int64_t nnz, cons
     if (o.l2_persist) CR_TRY(configure_l2_window(ctx));
 
     for (int n = 0; n < nmodes; ++n) {
-        int lanes, tile, red, batch_sh;
+        int lanes, tile, red;
+        ModeLayout h;  // the heuristic's shifts
         const int pi = o.pi_mode == CPAPR_PI_MATERIALISED ? 1 : o.pi_mode == CPAPR_PI_FUSED ? 0 : pi_auto(ctx);
-        heuristic_config(ctx, n, pi, &lanes, &tile, &red, &batch_sh);
+        heuristic_config(ctx, pi, h, &lanes, &tile, &red);
         if (o.rank_lanes) lanes = o.rank_lanes;
         if (o.tile_nnz) tile = o.tile_nnz;
         if (o.reduction) red = o.reduction;
         CR_TRY(configure_mode(ctx, n, lanes, tile, red));
-        if (!o.tile_nnz) ctx->mode[n].batch_sh = batch_sh;
+        if (!o.tile_nnz) {
+            ctx->mode[n].sh = h.sh;
+            ctx->mode[n].sh_df = h.sh_df;
+            ctx->mode[n].batch_sh = h.batch_sh;
+            CR_TRY(ensure_pair_storage(ctx));
+        }
         CR_TRY(configure_pi(ctx, n, pi));
     }
     if (o.autotune || o.tune_cache) CR_TRY(autotune(ctx));
@@ -568,6 +588,7 @@ cpapr_status cpapr_set_model(cpapr_ctx *ctx, const double *lambda, const double 
 cpapr_status cpapr_init_random(cpapr_ctx *ctx, uint64_t seed) {
     API_ENTER(ctx);
     CPAPR_TRY(launch_init_random(ctx, seed));
+    for (int m = 0; m < ctx->N; ++m) ctx->pair_state[m] = kPairStale;
     for (int m = 0; m < ctx->N; ++m)
         CPAPR_CUDA(ctx, cudaMemsetAsync(ctx->Phi[m], 0, (size_t)ctx->dims[m] * ctx->Rp * ctx->esize, ctx->stream));
     CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -674,7 +695,7 @@ cpapr_status cpapr_phi(cpapr_ctx *ctx, int32_t mode, const double *B, double *ou
     }
     // Phi[mode] holds the previous iteration's Phi that S reads: compute into
     // the separate output buffer instead.
-    CPAPR_TRY(launch_pi_build(ctx, mode));
+    CPAPR_TRY(prepare_phi(ctx, mode));
     CPAPR_TRY(launch_phi(ctx, mode, OP_PHI, ctx->B, ctx->outbuf, nullptr));
     CPAPR_TRY(download_matrix(ctx, ctx->outbuf, ctx->dims[mode], out));
     CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -737,10 +758,10 @@ cpapr_status cpapr_get_info(const cpapr_ctx *ctx, cpapr_info *info) {
     info->nnz = ctx->nnz;
     for (int m = 0; m < ctx->N; ++m) {
         info->dims[m] = ctx->dims[m];
-        info->tile_nnz[m] = ctx->mode[m].tile_nnz;
+        info->tile_nnz[m] = ctx->mode[m].tile_nnz << phi_shift(ctx, m);
         info->rank_lanes[m] = ctx->mode[m].lanes;
         info->reduction[m] = ctx->mode[m].reduction;
-        info->ntiles[m] = ctx->mode[m].ntiles;
+        info->ntiles[m] = (int32_t)ceil_div(ctx->nnz, info->tile_nnz[m]);
         info->nsplit[m] = ctx->mode[m].nsplit;
         info->pi_mode[m] = ctx->mode[m].pi ? CPAPR_PI_MATERIALISED : CPAPR_PI_FUSED;
     }

@@ -585,6 +585,7 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
     for (int i = 0; i < count; ++i) {
         CPAPR_CUDA(ctxs[i], cudaStreamSynchronize(ctxs[i]->stream));
         ctxs[i]->pi_mode_built = -1;  // the batched solve changes every factor
+        for (int m = 0; m < N; ++m) ctxs[i]->pair_state[m] = kPairStale;
     }
     // every tensor needs a rank class of the batched kernel and the segmented
     // reduction; it keeps its own tile size (tuned or heuristic) as long as
@@ -606,8 +607,15 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
             };
             while (sh > 0 && over(tile << sh)) --sh;
             while (tile > 256 && over(tile)) tile /= 2;
-            if (L.lanes != lanes || L.reduction != CPAPR_REDUCE_SEGMENTED || tile != L.tile_nnz)
+            if (L.lanes != lanes || L.reduction != CPAPR_REDUCE_SEGMENTED || tile != L.tile_nnz) {
+                const bool same = tile == L.tile_nnz;  // the context's own launches keep their tiles
+                const int s1 = L.sh, s2 = L.sh_df;
                 CPAPR_TRY(configure_mode(ctxs[i], n, lanes, tile, CPAPR_REDUCE_SEGMENTED));
+                if (same) {
+                    L.sh = s1;
+                    L.sh_df = s2;
+                }
+            }
             L.batch_sh = sh;
         }
         CPAPR_CUDA(ctxs[i], cudaStreamSynchronize(ctxs[i]->stream));
@@ -714,7 +722,7 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
             a.llpart = c->llpart;
             a.err = c->errflag + 3;
             a.stage_extra = injected_stage_shortfall();
-            a.dfdot = 0;  // the batched kernel keeps the FP64 dot (measured faster on the 64-tensor batch)
+            a.dfdot = 0;  // the batched kernel keeps FP64 rows and the FP64 dot
             // FP64 tensors whose mode n materialises its Khatri-Rao rows stream them here too
             if (sizeof(T) == 8 && L.pi && c->pibuf && c->nnz > 0) {
                 a.pi = c->pibuf;

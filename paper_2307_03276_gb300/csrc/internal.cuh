@@ -63,7 +63,9 @@ struct ModeLayout {
     int32_t *split = nullptr;      // [3 * nsplit] (row, first tile, last tile)
     int32_t *tsplit = nullptr;     // [ntiles] split of each tile's head partial, or -1
     int32_t *splitcnt = nullptr;   // [nsplit] partial counters of the tile kernel (zero between launches)
-    int32_t batch_sh = 0;          // the batched solver takes 2^batch_sh of these tiles as one (heuristic_config)
+    // a launch takes 2^k of these tiles as one (heuristic_config): k = sh, sh_df for
+    // the kernels over float pairs, batch_sh in the batched solver
+    int32_t sh = 0, sh_df = 0, batch_sh = 0;
     int32_t pi = 0;                // 1: Phi streams the materialised Khatri-Rao rows (built per outer iteration)
     int32_t nempty = 0;
     int32_t *erows = nullptr;      // [nempty] rows without nonzeros, increasing
@@ -93,6 +95,12 @@ struct cpapr_ctx {
     size_t factor_bytes = 0;
     cudaAccessPolicyWindow l2win{};  // persisting-L2 window over factor_block (num_bytes 0: none)
     void *B = nullptr;
+    // FP64 form, where a mode's Phi runs on float pairs (uses_pairs): the
+    // factors as pairs, their exponents, and which copies are current
+    float2 *P[CPAPR_MAX_MODES] = {};
+    int32_t *kexp = nullptr;                    // [N]
+    unsigned long long *pair_top = nullptr;     // [N] largest entries (scratch of launch_factor_pairs)
+    int pair_state[CPAPR_MAX_MODES] = {};       // kPairStale, kPairNormalised (stale, entries <= 1) or kPairCurrent
     // FP32 form: FP64 masters of the factors and of B.  The multiplicative
     // update, the shift S and the normalisation run on them in FP64 and
     // refresh the FP32 copies A[m] and B that Phi gathers, so an entry that
@@ -138,10 +146,16 @@ struct cpapr_ctx {
 namespace cpapr {
 
 constexpr int kColParts = 256;
+enum { kPairStale = 0, kPairNormalised = 1, kPairCurrent = 2 };
 // tiles from which an FP64 Phi launch takes the kernel with its dot on the FP32 pipe
 constexpr int kDfMinTiles = 152 * 4;
 // below this many tiles the automatic tile size shrinks (heuristic_config)
 constexpr int kSmallTiles = 152 * 4;
+// the kernels over float pairs: table tile, most nonzeros per group of lanes, and
+// fewest tiles a launch takes where it could take larger ones
+constexpr int kDfTile = 512;
+constexpr int kDfRun = 128;
+constexpr int kDfLaunchTiles = 152 * 9;
 
 // ---- error plumbing ------------------------------------------------------
 cpapr_status fail(cpapr_ctx *ctx, cpapr_status st, const std::string &msg);
@@ -196,8 +210,17 @@ enum PhiOp { OP_PHI = 0, OP_MTTKRP = 1, OP_LL = 2 };
 // B: I_n x Rp of the working type (ignored for MTTKRP).  inner: state whose
 // done flag / kkt slot the kernels use (may be null for a one-off Phi).
 cpapr_status launch_phi(cpapr_ctx *ctx, int n, PhiOp op, const void *B, void *out, InnerState *inner);
-// builds the materialised Khatri-Rao rows of mode n (a no-op unless the mode uses them)
-cpapr_status launch_pi_build(cpapr_ctx *ctx, int n);
+// does Phi of mode n run on float pairs (df_pair.cuh)?  Allocates their storage if so.
+bool uses_pairs(const cpapr_ctx *ctx, int n);
+// log2 of the table tiles per tile of mode n's Phi launch
+inline int phi_shift(const cpapr_ctx *ctx, int n) {
+    return uses_pairs(ctx, n) ? ctx->mode[n].sh_df : ctx->mode[n].sh;
+}
+cpapr_status ensure_pair_storage(cpapr_ctx *ctx);
+cpapr_status launch_factor_pairs(cpapr_ctx *ctx, int m, bool from_data);
+// what Phi of mode n reads besides the factors and B: the factors' pairs and
+// the materialised Khatri-Rao rows (each a no-op unless the mode uses them)
+cpapr_status prepare_phi(cpapr_ctx *ctx, int n);
 // selects the materialised (on = 1) or fused (0) Khatri-Rao rows for mode n
 cpapr_status configure_pi(cpapr_ctx *ctx, int n, int on);
 int pi_auto(const cpapr_ctx *ctx);

@@ -89,11 +89,12 @@ extern "C" cpapr_status cpapr_phi_noalloc(cpapr_ctx *ctx, int32_t mode, const do
     if (!out || !is_device_pointer(out)) return fail(ctx, CPAPR_E_ARG, "out must be a device pointer");
     if (B && !is_device_pointer(B)) return fail(ctx, CPAPR_E_ARG, "B must be NULL or a device pointer");
     const ModeLayout &L = ctx->mode[mode];
-    const int64_t need = (int64_t)2 * L.ntiles * ctx->Rp * (int64_t)ctx->esize;
+    const int64_t tiles = ceil_div(ctx->nnz, (int64_t)L.tile_nnz << phi_shift(ctx, mode));
+    const int64_t need = 2 * tiles * ctx->Rp * (int64_t)ctx->esize;
     if (need > (int64_t)CPAPR_NOALLOC_SCRATCH_BYTES)
         return fail(ctx, CPAPR_E_RANGE,
                     "cpapr_phi_noalloc: this mode needs " + std::to_string(need) + " bytes of scratch (2 x " +
-                        std::to_string(L.ntiles) + " tiles x " + std::to_string(ctx->Rp) +
+                        std::to_string(tiles) + " tiles x " + std::to_string(ctx->Rp) +
                         " ranks); the fixed scratch holds " + std::to_string((long long)CPAPR_NOALLOC_SCRATCH_BYTES) +
                         ": use cpapr_phi, or a larger tile_nnz");
     DeviceGuard guard(ctx->device);
@@ -112,7 +113,7 @@ extern "C" cpapr_status cpapr_phi_noalloc(cpapr_ctx *ctx, int32_t mode, const do
         // finishing tile reads is written earlier in this launch, so nothing
         // is cleared (the materialised rows, if the mode uses them, live in
         // the context's buffer and are rebuilt for this call)
-        CPAPR_TRY(launch_pi_build(ctx, mode));
+        CPAPR_TRY(prepare_phi(ctx, mode));
         CPAPR_TRY(launch_phi_given_carry(ctx, mode, ctx->B, ctx->outbuf, scratch));
         CPAPR_TRY(download_matrix(ctx, ctx->outbuf, ctx->dims[mode], out));
     }

@@ -17,6 +17,13 @@ cudaError_t launch_phi_f32_n2(const PhiArgs &, int, int, int, cudaStream_t, cons
 cudaError_t launch_phi_f32_n3(const PhiArgs &, int, int, int, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_phi_f32_n4(const PhiArgs &, int, int, int, cudaStream_t, const cudaAccessPolicyWindow *);
 
+cudaError_t launch_phi_df_n0(const PhiArgs &, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_phi_df_n2(const PhiArgs &, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_phi_df_n3(const PhiArgs &, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_phi_df_n4(const PhiArgs &, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_phi_df_pi(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_pi_pairs(const PhiArgs &, void *, cudaStream_t, const cudaAccessPolicyWindow *);
+
 bool phi_config_supported(int esize, int nm1, int rp, int lanes) {
     (void)nm1;
     if (lanes < 1 || rp % lanes) return false;
@@ -45,6 +52,15 @@ static cudaError_t dispatch(const cpapr_ctx *ctx, const PhiArgs &a, int rpl, int
     const int nm1 = ctx->N - 1;
     // Phi over materialised rows gathers no factor rows: no window
     const cudaAccessPolicyWindow *win = (op == OP_PHI && a.pi) ? nullptr : l2_window(ctx);
+    if (a.dfdot && a.pi && op != OP_MTTKRP) return launch_phi_df_pi(a, op, ctx->stream, win);
+    if (a.dfdot && op == OP_PHI) {
+        switch (nm1) {
+            case 2: return launch_phi_df_n2(a, ctx->stream, win);
+            case 3: return launch_phi_df_n3(a, ctx->stream, win);
+            case 4: return launch_phi_df_n4(a, ctx->stream, win);
+            default: return launch_phi_df_n0(a, ctx->stream, win);
+        }
+    }
     if (ctx->esize == 8) {
         switch (nm1) {
             case 2: return launch_phi_f64_n2(a, rpl, lanes, op, ctx->stream, win);
@@ -71,14 +87,50 @@ uint32_t injected_stage_shortfall() {
     return (s && s[0] == '1' && s[1] == 0) ? 16u : 0u;
 }
 
+// FP64 Phi on float pairs: accurate relative to max(s, eps) for the eps its
+// scales cover, and faster where the launch has at least a wave of tiles (4 per
+// SM); a launch of a few tiles is bound by one tile's latency, which the longer
+// FP32 instruction chains raise.
+bool uses_pairs(const cpapr_ctx *ctx, int n) {
+    const ModeLayout &L = ctx->mode[n];
+    const int dot = ctx->opt.fp64_dot;
+    return ctx->esize == 8 && ctx->nnz > 0 && ctx->Rp / L.lanes <= 8 && ctx->opt.eps >= 0x1p-43 &&
+           ctx->opt.eps <= 0x1p20 &&
+           (dot == CPAPR_DOT_FP32_PIPE ||
+            (dot == CPAPR_DOT_AUTO && ceil_div(ctx->nnz, (int64_t)L.tile_nnz << L.sh) >= kDfMinTiles));
+}
+
+cpapr_status ensure_pair_storage(cpapr_ctx *ctx) {
+    bool any = false;
+    for (int n = 0; n < ctx->N; ++n) any = any || uses_pairs(ctx, n);
+    if (!any || ctx->P[0]) return CPAPR_OK;
+    size_t ofs[CPAPR_MAX_MODES + 1] = {};
+    for (int m = 0; m < ctx->N; ++m) ofs[m + 1] = ofs[m] + (((size_t)ctx->dims[m] * ctx->Rp * 8 + 255) & ~(size_t)255);
+    void *p = nullptr;
+    CPAPR_TRY(dev_alloc(ctx, &p, ofs[ctx->N] + 256));
+    char *base = (char *)p;
+    ctx->pair_top = (unsigned long long *)(base + ofs[ctx->N]);
+    ctx->kexp = (int32_t *)(base + ofs[ctx->N] + 128);
+    for (int m = 0; m < ctx->N; ++m) {
+        ctx->P[m] = (float2 *)(base + ofs[m]);
+        ctx->pair_state[m] = kPairStale;
+    }
+    return CPAPR_OK;
+}
+
+// tiles of 2^sh table tiles
+static void set_tiles(PhiArgs &a, const ModeLayout &L, int sh) {
+    a.ksh = sh;
+    a.T = L.tile_nnz << sh;
+    a.ntiles = (int32_t)ceil_div(a.nnz, a.T);
+}
+
 static PhiArgs make_args(cpapr_ctx *ctx, int n, const void *B, void *out, InnerState *inner) {
     const ModeLayout &L = ctx->mode[n];
     PhiArgs a{};
     a.nnz = ctx->nnz;
-    a.T = L.tile_nnz;
-    a.ntiles = L.ntiles;
-    a.ksh = 0;
     a.ntab = L.ntiles;
+    set_tiles(a, L, L.sh);
     a.Rp = ctx->Rp;
     a.In = L.In;
     a.nm1 = ctx->N - 1;
@@ -108,15 +160,11 @@ static PhiArgs make_args(cpapr_ctx *ctx, int n, const void *B, void *out, InnerS
     a.llpart = ctx->llpart;
     a.err = ctx->errflag + 3;
     a.stage_extra = injected_stage_shortfall();
-    // FP64 Phi with its dot product on the FP32 pipe: accurate relative to
-    // max(s, eps) for eps >= 2^-43, and faster where the launch has at least a
-    // wave of tiles (4 per SM); a launch of a few tiles is bound by one
-    // tile's latency, which the longer FP32 instruction chains raise
-    const int dot = ctx->opt.fp64_dot;
-    a.dfdot = (ctx->esize == 8 && ctx->opt.eps >= 0x1p-43 &&
-               (dot == CPAPR_DOT_FP32_PIPE || (dot == CPAPR_DOT_AUTO && L.ntiles >= kDfMinTiles)))
-                  ? 1
-                  : 0;
+    a.dfdot = uses_pairs(ctx, n) ? 1 : 0;
+    a.mode = n;
+    a.kexp = ctx->kexp;
+    for (int m = 0, j = 0; m < ctx->N; ++m)
+        if (m != n) a.P[j++] = ctx->P[m];
     return a;
 }
 
@@ -193,14 +241,21 @@ static cudaError_t run_pi_build(const PhiArgs &a, T *pi, cudaStream_t s, const c
     }
 }
 
-cpapr_status launch_pi_build(cpapr_ctx *ctx, int n) {
+cpapr_status prepare_phi(cpapr_ctx *ctx, int n) {
+    if (uses_pairs(ctx, n))
+        for (int m = 0; m < ctx->N; ++m)
+            if (m != n && ctx->pair_state[m] != kPairCurrent) {
+                CPAPR_TRY(launch_factor_pairs(ctx, m, ctx->pair_state[m] == kPairStale));
+                ctx->pair_state[m] = kPairCurrent;
+            }
     if (!ctx->mode[n].pi || ctx->nnz == 0) return CPAPR_OK;
     if (!ctx->pibuf) return fail(ctx, CPAPR_E_STATE, "materialised Pi selected without its buffer");
     PhiArgs a = make_args(ctx, n, nullptr, nullptr, nullptr);
     ProfScope ps(ctx, K_PI);
     count_launch(ctx);
-    const cudaError_t e = ctx->esize == 8 ? run_pi_build<double>(a, (double *)ctx->pibuf, ctx->stream, l2_window(ctx))
-                                          : run_pi_build<float>(a, (float *)ctx->pibuf, ctx->stream, l2_window(ctx));
+    const cudaError_t e = a.dfdot           ? launch_pi_pairs(a, ctx->pibuf, ctx->stream, l2_window(ctx))
+                          : ctx->esize == 8 ? run_pi_build<double>(a, (double *)ctx->pibuf, ctx->stream, l2_window(ctx))
+                                            : run_pi_build<float>(a, (float *)ctx->pibuf, ctx->stream, l2_window(ctx));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "Pi build kernel");
     ctx->pi_mode_built = n;
     return CPAPR_OK;
@@ -211,6 +266,7 @@ cpapr_status launch_phi(cpapr_ctx *ctx, int n, PhiOp op, const void *B, void *ou
     const int64_t nel = (int64_t)L.In * ctx->Rp;
     PhiArgs a = make_args(ctx, n, B, out, inner);
     if (op == OP_PHI && L.pi) a.pi = ctx->pibuf;
+    if (op == OP_PHI) set_tiles(a, L, phi_shift(ctx, n));
     const bool atomic = a.atomic && op != OP_LL;
     if (ctx->nnz == 0 || atomic) {
         CPAPR_CUDA(ctx, cudaMemsetAsync(out, 0, (size_t)nel * ctx->esize, ctx->stream));
@@ -245,6 +301,7 @@ cpapr_status launch_phi_given_carry(cpapr_ctx *ctx, int n, const void *B, void *
     a.atomic = 0;
     a.carry = carry;
     if (L.pi) a.pi = ctx->pibuf;
+    set_tiles(a, L, phi_shift(ctx, n));
     if (ctx->nnz == 0) return fail(ctx, CPAPR_E_ARG, "empty tensor");
     CPAPR_TRY(launch_zero_empty(ctx, n, out));
     cudaError_t e = dispatch(ctx, a, ctx->Rp / L.lanes, L.lanes, OP_PHI);
@@ -269,13 +326,16 @@ cpapr_status launch_loglik(cpapr_ctx *ctx, double *dst) {
     CPAPR_TRY(launch_scale_b(ctx, n, ctx->B));
     PhiArgs a = make_args(ctx, n, ctx->B, nullptr, nullptr);
     a.atomic = 0;
-    if (use_pi) a.pi = ctx->pibuf;
+    if (use_pi) {
+        a.pi = ctx->pibuf;
+        set_tiles(a, L, phi_shift(ctx, n));
+    }
     {
         ProfScope ps(ctx, K_LL);
         cudaError_t e = dispatch(ctx, a, ctx->Rp / L.lanes, L.lanes, OP_LL);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "log-likelihood kernel");
         count_launch(ctx);
-        CPAPR_TRY(launch_ll_total(ctx, ctx->llpart, L.ntiles, dst));
+        CPAPR_TRY(launch_ll_total(ctx, ctx->llpart, a.ntiles, dst));
     }
     return CPAPR_OK;
 }

@@ -93,7 +93,7 @@ static cpapr_status enqueue_mode(cpapr_ctx *ctx, int n, double tol, int max_inne
     CPAPR_TRY(launch_empty_kkt(ctx, n, ctx->B, inner));
     // the other modes' factors are fixed for this inner loop: their
     // Khatri-Rao rows are built once here if the mode streams them
-    CPAPR_TRY(launch_pi_build(ctx, n));
+    CPAPR_TRY(prepare_phi(ctx, n));
     if (ctx->opt.use_graph) {
         CPAPR_TRY(build_inner_graph(ctx, n, tol, max_inner));
         CPAPR_CUDA(ctx, cudaGraphLaunch(ctx->graph_exec[n], ctx->stream));
@@ -357,7 +357,7 @@ cpapr_status autotune(cpapr_ctx *ctx) {
                     const int pi = cand / 2;
                     CPAPR_TRY(configure_mode(ctx, n, lanes, tile, red));
                     CPAPR_TRY(configure_pi(ctx, n, pi));
-                    if (pi) CPAPR_TRY(launch_pi_build(ctx, n));
+                    CPAPR_TRY(prepare_phi(ctx, n));
                     // a fresh inner state: not done, violation slots clear
                     CPAPR_CUDA(ctx, cudaMemsetAsync(inner, 0, sizeof(InnerState), ctx->stream));
                     CPAPR_TRY(launch_phi(ctx, n, OP_PHI, ctx->B, ctx->outbuf, inner));
