@@ -220,7 +220,6 @@ static void heuristic_config(const cpapr_ctx *ctx, int pi, ModeLayout &L, int *l
     // walk saves (1e5 at 64: 51 us, 1e6: 290).  The batched solver, whose launch
     // holds the tiles of many tensors, keeps the large ones (64 tensors 80 ms, 91
     // in these small ones).
-    // FP32 keeps one tile size whatever the tensor's: its sums keep their order.
     const bool f64 = ctx->esize == 8;
     const int full = *tile;
     L.sh = L.sh_df = L.batch_sh = 0;
@@ -240,9 +239,18 @@ static void heuristic_config(const cpapr_ctx *ctx, int pi, ModeLayout &L, int *l
                ceil_div(ctx->nnz, (int64_t)*tile << (L.sh_df + 1)) >= kDfLaunchTiles)
             ++L.sh_df;
     }
-    while (f64 && *tile > 64 && ceil_div(ctx->nnz, *tile / 2) < kSmallTiles) {
+    // FP32: at most one tile per SM below 1024 nonzeros, one and a half where eight or
+    // more lanes per nonzero make long runs (1e4 nonzeros, R = 16: 34 -> 15 us; 1e5: 32 ->
+    // 24; R = 32: 39 -> 28); 2048 only from 4 tiles per SM on, or 8.  The batched solver
+    // takes the same tiles, so that a tensor's FP32 sums keep one order in both,
+    // and larger numbers of them cost it more than a lone launch gains (64 tensors:
+    // 27.5 ms at one tile per SM, 34 at four).
+    const bool wide = g >= 8;
+    while (!f64 && *tile > 1024 && ceil_div(ctx->nnz, *tile / 2) < (wide ? 2 : 1) * kSmallTiles) *tile /= 2;
+    const int few = f64 ? kSmallTiles : wide ? kSmallTiles * 3 / 8 : kSmallTiles / 4;
+    while (*tile > 64 && ceil_div(ctx->nnz, *tile / 2) < few) {
         *tile /= 2;
-        ++L.batch_sh;
+        L.batch_sh += f64 ? 1 : 0;
     }
     *reduction = CPAPR_REDUCE_SEGMENTED;
 }

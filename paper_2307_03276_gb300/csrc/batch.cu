@@ -26,6 +26,7 @@
 #include <mutex>
 #include <vector>
 
+#include "direct.cuh"
 #include "ll_total.cuh"
 #include "phi_kernels.cuh"
 
@@ -88,17 +89,35 @@ __host__ __device__ constexpr int batch_unroll() {
 }
 
 template <typename T> __host__ __device__ constexpr int batch_threads() { return sizeof(T) == 8 ? 128 : 256; }
+// the FP32 Phi runs the direct tile (direct.cuh), as the single-tensor launch does
+template <typename T, int OP> __host__ __device__ constexpr bool batch_direct() { return sizeof(T) == 4 && OP == OP_PHI; }
+template <typename T, int OP> __host__ __device__ constexpr int batch_block() {
+    return batch_direct<T, OP>() ? kDirectThreads : batch_threads<T>();
+}
 // resident blocks per SM the registers are held to (measured on GB300): the
 // FP32 classes all keep one float4 per lane, like the single-tensor kernel's
 // four-block case; every FP64 class fits three blocks (168 registers)
-template <typename T> __host__ __device__ constexpr int batch_min_blocks() { return sizeof(T) == 8 ? 3 : 4; }
+template <typename T, int OP = OP_LL> __host__ __device__ constexpr int batch_min_blocks() {
+    return batch_direct<T, OP>() ? 6 : sizeof(T) == 8 ? 3 : 4;
+}
+
+// One class's direct tile as a function of its own: four of them inlined side by
+// side spilled 432 bytes at 64 registers, each alone none.
+template <int NM1, int G, int OP, bool PI>
+__device__ __noinline__ void direct_class(const PhiArgs &a, int tile, unsigned char *smem, double *red) {
+    direct_tile<NM1, G, OP, PI>(a, tile, smem, red);
+}
 
 template <typename T, int NM1, int K, int OP, bool PI = false>
 __device__ __forceinline__ bool run_class(const PhiArgs &a, int tile, unsigned char *smem, double *red, uint64_t *bar,
                                           uint32_t &phase) {
     constexpr int RPL = Classes<T>::rpl[K];
     constexpr int G = Classes<T>::g[K];
-    return phi_tile_body<T, NM1, RPL, G, OP, batch_threads<T>(), batch_unroll<T, RPL, G>(), PI>(a, tile, smem, red,
+    if constexpr (batch_direct<T, OP>()) {
+        direct_class<NM1, G, OP, PI>(a, tile, smem, red);
+        return true;
+    } else
+        return phi_tile_body<T, NM1, RPL, G, OP, batch_threads<T>(), batch_unroll<T, RPL, G>(), PI>(a, tile, smem, red,
                                                                                                bar, phase);
 }
 
@@ -122,11 +141,10 @@ __device__ __forceinline__ bool run_item(const PhiArgs &a, int cfg, int tile, un
 // OP_PHI: Phi of every listed tile; OP_LL: the tile sums of x log m (the
 // descriptors then carry the scaled mode-0 B and no inner-loop state).
 template <typename T, int NM1, int OP = OP_PHI>
-__global__ void __launch_bounds__(batch_threads<T>(), batch_min_blocks<T>()) batch_phi_kernel(const BatchTensor *__restrict__ desc,
-                                                                       const int2 *__restrict__ items, int nitems,
-                                                                       BatchCtl *ctl) {
+__global__ void __launch_bounds__(batch_block<T, OP>(), batch_min_blocks<T, OP>())
+    batch_phi_kernel(const BatchTensor *__restrict__ desc, const int2 *__restrict__ items, int nitems, BatchCtl *ctl) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ double red[batch_threads<T>() / 32];
+    __shared__ double red[batch_block<T, OP>() / 32];
     __shared__ int s_item;
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) stage_barrier_init(&bar);
@@ -140,6 +158,17 @@ __global__ void __launch_bounds__(batch_threads<T>(), batch_min_blocks<T>()) bat
         __syncthreads();
         if (it >= nitems) break;
         const int2 w = items[it];
+        if constexpr (batch_direct<T, OP>()) {
+            // the tile reads its arguments from shared memory (the previous
+            // item's last reads are behind the barriers above)
+            __shared__ PhiArgs s_a;
+            static_assert(sizeof(PhiArgs) % 4 == 0, "copied by words");
+            for (int k = threadIdx.x; k < (int)(sizeof(PhiArgs) / 4); k += batch_block<T, OP>())
+                reinterpret_cast<uint32_t *>(&s_a)[k] = reinterpret_cast<const uint32_t *>(&desc[w.x].a)[k];
+            __syncthreads();
+            if (!s_a.inner->done) run_item<T, NM1, OP, false>(s_a, desc[w.x].cfg, w.y, smem_raw, red, &bar, phase);
+            continue;
+        }
         const PhiArgs a = desc[w.x].a;
         if constexpr (sizeof(T) == 8 && OP == OP_PHI) {
             if (a.pi) {
@@ -454,10 +483,10 @@ Plan *g_cache = nullptr;
 
 template <typename T>
 cudaError_t launch_phi_batch(const ModePlan &mp, int nm1, int grid, BatchCtl *ctl, cudaStream_t s) {
-    const size_t smem = mp.smem;
+    const size_t smem = batch_direct<T, OP_PHI>() ? direct_smem() : mp.smem;
     auto go = [&](auto kern) {
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        kern<<<grid, batch_threads<T>(), smem, s>>>(mp.desc, mp.tiles, mp.ntiles, ctl);
+        kern<<<grid, batch_block<T, OP_PHI>(), smem, s>>>(mp.desc, mp.tiles, mp.ntiles, ctl);
         return cudaGetLastError();
     };
     switch (nm1) {
@@ -497,6 +526,7 @@ cudaError_t launch_pi_batch(const ModePlan &mp, int nm1, const int32_t *flags, c
 
 template <typename T>
 int persistent_grid(int nm1, size_t smem) {
+    if (batch_direct<T, OP_PHI>()) smem = direct_smem();
     int dev = 0, sms = 152, per = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -504,7 +534,7 @@ int persistent_grid(int nm1, size_t smem) {
                              : nm1 == 3 ? (const void *)batch_phi_kernel<T, 3>
                                         : nm1 == 4 ? (const void *)batch_phi_kernel<T, 4> : (const void *)batch_phi_kernel<T, 0>;
     if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, batch_threads<T>(), smem) != cudaSuccess || per < 1)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, batch_block<T, OP_PHI>(), smem) != cudaSuccess || per < 1)
         per = 1;
     cudaGetLastError();
     return sms * per;

@@ -37,7 +37,7 @@
 // smaller than with the FP64 scale-add and the one-step quotient it replaces.
 #pragma once
 
-#include "phi_kernels.cuh"
+#include "direct.cuh"
 
 namespace cpapr {
 
@@ -320,30 +320,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
     auto bit_at = [&](int p) -> uint32_t { return (__ldg(a.rstart + (p >> 5)) >> (p & 31)) & 1u; };
     auto col = [&](int v) -> int { return (v * G + lane) * 2; };
 
-    // index in nzrow of the row holding qa: the tile's first row plus the row
-    // starts in (p0, qa], counted by the warp over the tile's words
-    int kcur = __ldg(a.krow + ((int64_t)t << a.ksh));
-    {
-        const int w0 = p0 >> 5, w1 = p1 >> 5, wt = qa >> 5;
-        int before = 0;
-        for (int base = w0; base <= w1; base += 32) {
-            const int w = base + wlane;
-            uint32_t b = w <= w1 ? __ldg(a.rstart + w) : 0u;
-            if (w == w0) b &= ~((2u << (p0 & 31)) - 1u);
-            const int c = __popc(b);
-            int x = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(full, x, o);
-                if (wlane >= o) x += y;
-            }
-            const int src = wt - base;
-            const int ex = __shfl_sync(full, x - c, src & 31);
-            const uint32_t bw = __shfl_sync(full, b, src & 31);
-            if (src >= 0 && src < 32) kcur += before + ex + __popc(bw & (0xffffffffu >> (31 - (qa & 31))));
-            before += __shfl_sync(full, x, 31);
-        }
-    }
+    int kcur = run_first_row(a, t, p0, p1, qa, wlane);
     const bool run = qa < qb;
     const bool head_open = qa > 0 && !bit_at(qa);
     const bool tail_open = qb < a.nnz && !bit_at(qb);

@@ -22,6 +22,11 @@ cudaError_t launch_phi_df_n2(const PhiArgs &, cudaStream_t, const cudaAccessPoli
 cudaError_t launch_phi_df_n3(const PhiArgs &, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_phi_df_n4(const PhiArgs &, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_phi_df_pi(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_direct_f32_n0(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_direct_f32_n2(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_direct_f32_n3(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_direct_f32_n4(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_direct_f32_pi(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_pi_pairs(const PhiArgs &, void *, cudaStream_t, const cudaAccessPolicyWindow *);
 
 bool phi_config_supported(int esize, int nm1, int rp, int lanes) {
@@ -59,6 +64,15 @@ static cudaError_t dispatch(const cpapr_ctx *ctx, const PhiArgs &a, int rpl, int
             case 3: return launch_phi_df_n3(a, ctx->stream, win);
             case 4: return launch_phi_df_n4(a, ctx->stream, win);
             default: return launch_phi_df_n0(a, ctx->stream, win);
+        }
+    }
+    if (ctx->esize == 4 && op != OP_LL && !(op == OP_MTTKRP && nm1 == 2)) {
+        if (a.pi) return launch_direct_f32_pi(a, op, ctx->stream, win);
+        switch (nm1) {
+            case 2: return launch_direct_f32_n2(a, op, ctx->stream, win);
+            case 3: return launch_direct_f32_n3(a, op, ctx->stream, win);
+            case 4: return launch_direct_f32_n4(a, op, ctx->stream, win);
+            default: return launch_direct_f32_n0(a, op, ctx->stream, win);
         }
     }
     if (ctx->esize == 8) {

@@ -29,11 +29,11 @@ def max_rel(got, want):
 
 
 # (nonzeros, expected tile): FP64 takes the smallest power of two >= 64 with
-# fewer than 608 tiles, FP32 keeps its tile
+# fewer than 608 tiles, FP32 with fewer than 152
 @pytest.mark.parametrize("precision,nnz,tile", [
     (cpapr.CPAPR_FP64, 1, 64), (cpapr.CPAPR_FP64, 63, 64), (cpapr.CPAPR_FP64, 64 * 607, 64),
     (cpapr.CPAPR_FP64, 64 * 607 + 1, 128), (cpapr.CPAPR_FP64, 128 * 607 + 1, 256),
-    (cpapr.CPAPR_FP32, 1, 2048), (cpapr.CPAPR_FP32, 40_000, 2048)])
+    (cpapr.CPAPR_FP32, 1, 64), (cpapr.CPAPR_FP32, 64 * 151, 64), (cpapr.CPAPR_FP32, 64 * 151 + 1, 128)])
 def test_small_tiles_match_oracle(precision, nnz, tile):
     dims, idx, vals = heavy_row_tensor(nnz, nnz)
     fs = synth.random_factors(dims, 10, 3)
