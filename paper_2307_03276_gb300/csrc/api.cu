@@ -107,6 +107,51 @@ cpapr_status dev_alloc(cpapr_ctx *ctx, void **p, size_t bytes) {
     return CPAPR_OK;
 }
 
+// Slots of page-locked memory come from blocks of 64; a block whose slots are all
+// free is given back unless it is the only such one.
+namespace {
+struct SlotBlock {
+    HostSlot *base;
+    uint64_t used;
+};
+std::mutex g_slot_mu;
+std::vector<SlotBlock> g_slots;
+}  // namespace
+
+HostSlot *host_slot_acquire() {
+    std::lock_guard<std::mutex> lock(g_slot_mu);
+    for (SlotBlock &b : g_slots)
+        if (b.used != ~0ull) {
+            const int k = __builtin_ctzll(~b.used);
+            b.used |= 1ull << k;
+            return b.base + k;
+        }
+    void *p = nullptr;
+    if (cudaHostAlloc(&p, 64 * sizeof(HostSlot), cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    g_slots.push_back({static_cast<HostSlot *>(p), 1ull});
+    return static_cast<HostSlot *>(p);
+}
+
+void host_slot_release(HostSlot *s) {
+    if (!s) return;
+    std::lock_guard<std::mutex> lock(g_slot_mu);
+    int spare = 0;
+    for (const SlotBlock &b : g_slots) spare += b.used == 0 ? 1 : 0;
+    for (size_t i = 0; i < g_slots.size(); ++i) {
+        SlotBlock &b = g_slots[i];
+        if (s < b.base || s >= b.base + 64) continue;
+        b.used &= ~(1ull << (s - b.base));
+        if (b.used == 0 && spare > 0) {
+            cudaFreeHost(b.base);
+            g_slots.erase(g_slots.begin() + (std::ptrdiff_t)i);
+        }
+        return;
+    }
+}
+
 void count_launch(cpapr_ctx *ctx, int k) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(ctx->stream, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone) {
@@ -412,6 +457,7 @@ void cpapr_destroy(cpapr_ctx *ctx) {
     }
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
+    host_slot_release(ctx->host);
     delete ctx;
 }
 
@@ -477,6 +523,8 @@ cpapr_status cpapr_create(int32_t nmodes, const int64_t *dims, int64_t nnz, cons
         st = (expr);                     \
         if (st != CPAPR_OK) return bail(st); \
     } while (0)
+    ctx->host = host_slot_acquire();
+    if (!ctx->host) return bail(fail(ctx, CPAPR_E_NOMEM, "page-locked host allocation failed"));
     CR_TRY(dev_alloc(ctx, &p, 64));
     ctx->errflag = (int32_t *)p;
     CR_TRY(dev_alloc(ctx, &p, sizeof(InnerState) * nmodes));
@@ -570,21 +618,16 @@ cpapr_status cpapr_set_model(cpapr_ctx *ctx, const double *lambda, const double 
     if (!lambda || !factors) return fail(ctx, CPAPR_E_ARG, "lambda or factors is NULL");
     for (int m = 0; m < ctx->N; ++m)
         if (!factors[m]) return fail(ctx, CPAPR_E_ARG, "factors[m] is NULL");
-    std::vector<double> hl(ctx->Rp, 0.0);
-    CPAPR_CUDA(ctx, cudaMemcpy(hl.data(), lambda, (size_t)ctx->R * 8, cudaMemcpyDefault));
-    for (int r = 0; r < ctx->R; ++r)
-        if (!(hl[r] >= 0.0) || std::isinf(hl[r])) return fail(ctx, CPAPR_E_VALUE, "lambda must be finite and >= 0");
+    int32_t *flags = ctx->host->flags;
     CPAPR_CUDA(ctx, cudaMemsetAsync(ctx->errflag, 0, 16, ctx->stream));
-    CPAPR_CUDA(ctx, cudaMemcpyAsync(ctx->lambda, hl.data(), (size_t)ctx->Rp * 8, cudaMemcpyHostToDevice, ctx->stream));
-    for (int m = 0; m < ctx->N; ++m) {
-        CPAPR_TRY(upload_factor(ctx, m, factors[m]));
-        CPAPR_CUDA(ctx, cudaMemsetAsync(ctx->Phi[m], 0, (size_t)ctx->dims[m] * ctx->Rp * ctx->esize, ctx->stream));
-    }
-    int32_t flags[4] = {0, 0, 0, 0};
+    CPAPR_TRY(launch_set_model(ctx, lambda, factors));
     CPAPR_CUDA(ctx, cudaMemcpyAsync(flags, ctx->errflag, 16, cudaMemcpyDeviceToHost, ctx->stream));
     CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    // a bad lambda leaves the model as it was
+    if (flags[0]) return fail(ctx, CPAPR_E_VALUE, "lambda must be finite and >= 0");
     ctx->k_total = 0;
     ctx->pi_mode_built = -1;
+    for (int m = 0; m < ctx->N; ++m) ctx->pair_state[m] = kPairStale;
     if (flags[2]) {
         ctx->model_set = false;
         return fail(ctx, CPAPR_E_VALUE, "factor entries must be finite and >= 0");
@@ -620,8 +663,6 @@ cpapr_status cpapr_get_model(cpapr_ctx *ctx, double *lambda, double *const *fact
                                                   ctx->stream));
             else
                 CPAPR_TRY(download_matrix(ctx, ctx->A[m], ctx->dims[m], factors[m]));
-            // download_matrix stages FP32 through ctx->stage: finish before reuse
-            CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         }
     CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     return CPAPR_OK;
@@ -635,8 +676,8 @@ cpapr_status cpapr_get_state(cpapr_ctx *ctx, double *lambda, double *const *fact
         for (int m = 0; m < ctx->N; ++m) {
             if (!phi_prev[m]) continue;
             CPAPR_TRY(download_matrix(ctx, ctx->Phi[m], ctx->dims[m], phi_prev[m]));
-            CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         }
+    CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
     if (outer_done) *outer_done = ctx->k_total;
     return CPAPR_OK;
 }
@@ -667,14 +708,18 @@ cpapr_status cpapr_set_state(cpapr_ctx *ctx, const double *lambda, const double 
     return CPAPR_OK;
 }
 
-// After a call's last synchronisation: did a bounded device-side wait give
-// up?  (errflag[3]; a call without one, such as cpapr_phi_noalloc, leaves it
-// for the next call that checks.)
-static cpapr_status check_waits(cpapr_ctx *ctx) {
-    int32_t f = 0;
-    CPAPR_CUDA(ctx, cudaMemcpyAsync(&f, ctx->errflag + 3, 4, cudaMemcpyDeviceToHost, ctx->stream));
+// The flag of the bounded device-side waits (errflag[3]) on its way to the host,
+// behind a call's other work.
+static cpapr_status fetch_waits(cpapr_ctx *ctx) {
+    CPAPR_CUDA(ctx, cudaMemcpyAsync(&ctx->host->flags[3], ctx->errflag + 3, 4, cudaMemcpyDeviceToHost, ctx->stream));
+    return CPAPR_OK;
+}
+
+// A call's last synchronisation, after fetch_waits: did a wait give up?  (A call
+// without one, such as cpapr_phi_noalloc, leaves the flag for the next that checks.)
+static cpapr_status finish_waits(cpapr_ctx *ctx) {
     CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    if (!f) return CPAPR_OK;
+    if (!ctx->host->flags[3]) return CPAPR_OK;
     CPAPR_CUDA(ctx, cudaMemsetAsync(ctx->errflag + 3, 0, 4, ctx->stream));
     // tiles that gave up never counted their partials: clear the counters
     for (int n = 0; n < ctx->N; ++n)
@@ -706,8 +751,8 @@ cpapr_status cpapr_phi(cpapr_ctx *ctx, int32_t mode, const double *B, double *ou
     CPAPR_TRY(prepare_phi(ctx, mode));
     CPAPR_TRY(launch_phi(ctx, mode, OP_PHI, ctx->B, ctx->outbuf, nullptr));
     CPAPR_TRY(download_matrix(ctx, ctx->outbuf, ctx->dims[mode], out));
-    CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return check_waits(ctx);
+    CPAPR_TRY(fetch_waits(ctx));
+    return finish_waits(ctx);
 }
 
 cpapr_status cpapr_mttkrp(cpapr_ctx *ctx, int32_t mode, double *out) {
@@ -716,8 +761,8 @@ cpapr_status cpapr_mttkrp(cpapr_ctx *ctx, int32_t mode, double *out) {
     if (!out) return fail(ctx, CPAPR_E_ARG, "out is NULL");
     CPAPR_TRY(launch_phi(ctx, mode, OP_MTTKRP, nullptr, ctx->outbuf, nullptr));
     CPAPR_TRY(download_matrix(ctx, ctx->outbuf, ctx->dims[mode], out));
-    CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return check_waits(ctx);
+    CPAPR_TRY(fetch_waits(ctx));
+    return finish_waits(ctx);
 }
 
 cpapr_status cpapr_loglik(cpapr_ctx *ctx, double *out) {
@@ -726,8 +771,8 @@ cpapr_status cpapr_loglik(cpapr_ctx *ctx, double *out) {
     if (!ctx->model_set) return fail(ctx, CPAPR_E_STATE, "no model set");
     CPAPR_TRY(launch_loglik(ctx, ctx->scalars));
     CPAPR_CUDA(ctx, cudaMemcpyAsync(out, ctx->scalars, 8, cudaMemcpyDefault, ctx->stream));
-    CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    return check_waits(ctx);
+    CPAPR_TRY(fetch_waits(ctx));
+    return finish_waits(ctx);
 }
 
 cpapr_status cpapr_mu_solve(cpapr_ctx *ctx, double tol, int32_t max_outer, int32_t max_inner, cpapr_result *res,
@@ -737,7 +782,8 @@ cpapr_status cpapr_mu_solve(cpapr_ctx *ctx, double tol, int32_t max_outer, int32
     if (max_outer < 0 || max_inner < 1 || !(tol >= 0.0)) return fail(ctx, CPAPR_E_ARG, "bad tol / iteration bounds");
     if (!ctx->model_set) return fail(ctx, CPAPR_E_STATE, "no model set");
     CPAPR_TRY(mu_solve(ctx, tol, max_outer, max_inner, res, inner_trace, ll_trace, kkt_trace));
-    return check_waits(ctx);
+    // (mu_solve fetched the flag with the log-likelihood)
+    return finish_waits(ctx);
 }
 
 cpapr_status cpapr_batch_mu_solve(cpapr_ctx *const *ctxs, int32_t count, double tol, int32_t max_outer,
@@ -752,7 +798,8 @@ cpapr_status cpapr_batch_mu_solve(cpapr_ctx *const *ctxs, int32_t count, double 
     if (max_outer < 0 || max_inner < 1 || !(tol >= 0.0)) return fail(nullptr, CPAPR_E_ARG, "bad tol / iteration bounds");
     const cpapr_status st = batch_mu_solve(ctxs, count, tol, max_outer, max_inner, results);
     if (st != CPAPR_OK) return st;
-    for (int i = 0; i < count; ++i) CPAPR_TRY(check_waits(ctxs[i]));
+    for (int i = 0; i < count; ++i) CPAPR_TRY(fetch_waits(ctxs[i]));
+    for (int i = 0; i < count; ++i) CPAPR_TRY(finish_waits(ctxs[i]));
     return CPAPR_OK;
 }
 

@@ -47,6 +47,17 @@ struct InnerState {
     double viol;        // last checked violation
 };
 
+// What a context reads back from the device, in page-locked memory: a copy into
+// it is asynchronous, so that one synchronisation serves a call's results, inner
+// states and error flags (a copy into pageable memory waits by itself).
+struct HostSlot {
+    InnerState inner[kMaxModes];
+    double ll;
+    int32_t flags[4];
+};
+HostSlot *host_slot_acquire();  // null if none can be had
+void host_slot_release(HostSlot *s);
+
 struct ModeLayout {
     int32_t In = 0;
     int32_t *seg = nullptr;
@@ -123,6 +134,7 @@ struct cpapr_ctx {
     cpapr::InnerState *inner = nullptr;  // [N]
     double *scalars = nullptr;   // misc device scalars
     int32_t *errflag = nullptr;  // device error flags
+    cpapr::HostSlot *host = nullptr;
     bool model_set = false;
     int64_t k_total = 0;
     bool sticky = false;
@@ -252,6 +264,10 @@ cpapr_status upload_matrix(cpapr_ctx *ctx, const double *src, int64_t rows, void
 // factor m from the caller's rows x R doubles (and its FP64 master in the FP32 form)
 cpapr_status upload_factor(cpapr_ctx *ctx, int m, const double *src);
 cpapr_status download_matrix(cpapr_ctx *ctx, const void *src, int64_t rows, double *dst); // Rp cols T -> R cols
+// lambda and every factor from the caller's memory, Phi cleared (launches and copies only)
+cpapr_status launch_set_model(cpapr_ctx *ctx, const double *lambda, const double *const *factors);
+// memory of the context's device (or managed) that a kernel may read or write as doubles in place
+bool device_doubles(const cpapr_ctx *ctx, const void *p);
 cpapr_status launch_kkt_rows(cpapr_ctx *ctx, int n, const void *B, const void *Phi, InnerState *inner);
 
 // ---- small utilities (index.cu) ---------------------------------------------

@@ -406,10 +406,106 @@ __global__ void convert_kernel(const double *__restrict__ src, T *__restrict__ d
     }
 }
 
+// rows x R doubles out of a padded matrix
 template <typename T>
-__global__ void widen_kernel(const T *__restrict__ src, double *__restrict__ dst, int64_t n) {
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-        dst[e] = (double)src[e];
+__global__ void widen_kernel(const T *__restrict__ src, double *__restrict__ dst, int64_t n, int R, int lg) {
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        const int c = (int)(e & ((1 << lg) - 1));
+        if (c < R) dst[(e >> lg) * R + c] = (double)src[e];
+    }
+}
+
+// A model in one launch: every block checks lambda (a bad one leaves everything as
+// it was, errflag[0]); factor m's rows x R doubles, read in place, become its
+// padded copy (and master), checked (errflag[2]); its Phi is cleared.
+struct ModelArgs {
+    const double *lambda_src;
+    double *lambda;
+    const double *src[kMaxModes];
+    void *A[kMaxModes], *Phi[kMaxModes];
+    double *A64[kMaxModes];
+    int64_t e0[kMaxModes + 1];  // first padded element of each listed factor
+    int n, R, Rp, lg;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(256) set_model_kernel(const ModelArgs a, int32_t *__restrict__ errflag) {
+    const double l = (int)threadIdx.x < a.R ? a.lambda_src[threadIdx.x] : 0.0;
+    if (__syncthreads_or(!(l >= 0.0) || isinf(l))) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) errflag[0] = 1;
+        return;
+    }
+    if (blockIdx.x == 0 && (int)threadIdx.x < a.Rp) a.lambda[threadIdx.x] = l;
+    const int64_t total = a.e0[a.n];
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        int m = 0;
+        while (m + 1 < a.n && e >= a.e0[m + 1]) ++m;
+        const int64_t k = e - a.e0[m];
+        const int c = (int)(k & (a.Rp - 1));  // Rp is a power of two
+        const double v = c < a.R ? a.src[m][(k >> a.lg) * a.R + c] : 0.0;
+        if (!(v >= 0.0) || isinf(v)) atomicOr(errflag + 2, 1);
+        if (a.A64[m]) a.A64[m][k] = v;
+        reinterpret_cast<T *>(a.A[m])[k] = (T)v;
+        reinterpret_cast<T *>(a.Phi[m])[k] = T(0);
+    }
+}
+
+bool device_doubles(const cpapr_ctx *ctx, const void *p) {
+    cudaPointerAttributes t;
+    if (cudaPointerGetAttributes(&t, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    // (another device's memory, like the host's, goes through a copy)
+    return ((t.type == cudaMemoryTypeDevice && t.device == ctx->device) || t.type == cudaMemoryTypeManaged) &&
+           ((uintptr_t)p & 7) == 0;
+}
+
+cpapr_status launch_set_model(cpapr_ctx *ctx, const double *lambda, const double *const *factors) {
+    ModelArgs a{};
+    a.R = ctx->R;
+    a.Rp = ctx->Rp;
+    while ((1 << a.lg) < ctx->Rp) ++a.lg;
+    a.lambda = ctx->lambda;
+    a.lambda_src = lambda;
+    if (!device_doubles(ctx, lambda)) {
+        // (colsum: N x Rp doubles of scratch)
+        CPAPR_CUDA(ctx, cudaMemcpyAsync(ctx->colsum, lambda, (size_t)ctx->R * 8, cudaMemcpyDefault, ctx->stream));
+        a.lambda_src = ctx->colsum;
+    }
+    auto go = [&]() -> cpapr_status {
+        if (a.n == 0) return CPAPR_OK;
+        count_launch(ctx);
+        const unsigned grid = grid_for(a.e0[a.n]);
+        if (ctx->esize == 8)
+            set_model_kernel<double><<<grid, 256, 0, ctx->stream>>>(a, ctx->errflag);
+        else
+            set_model_kernel<float><<<grid, 256, 0, ctx->stream>>>(a, ctx->errflag);
+        CPAPR_CUDA(ctx, cudaGetLastError());
+        a.n = 0;
+        return CPAPR_OK;
+    };
+    // factors in device memory together; each other one through the staging buffer
+    for (int pass = 0; pass < 2; ++pass) {
+        for (int m = 0; m < ctx->N; ++m) {
+            const bool dev = device_doubles(ctx, factors[m]);
+            if (dev != (pass == 0)) continue;
+            a.src[a.n] = factors[m];
+            if (!dev) {
+                CPAPR_CUDA(ctx, cudaMemcpyAsync(ctx->stage, factors[m], (size_t)ctx->dims[m] * ctx->R * 8,
+                                                cudaMemcpyDefault, ctx->stream));
+                a.src[a.n] = ctx->stage;
+            }
+            a.A[a.n] = ctx->A[m];
+            a.A64[a.n] = ctx->A64[m];
+            a.Phi[a.n] = ctx->Phi[m];
+            a.e0[a.n + 1] = a.e0[a.n] + ctx->dims[m] * ctx->Rp;
+            ++a.n;
+            if (!dev) CPAPR_TRY(go());
+        }
+        CPAPR_TRY(go());
+    }
+    return CPAPR_OK;
 }
 
 static cpapr_status upload_matrix2(cpapr_ctx *ctx, const double *src, int64_t rows, void *dst, double *dst64) {
@@ -442,16 +538,22 @@ cpapr_status upload_factor(cpapr_ctx *ctx, int m, const double *src) {
 cpapr_status download_matrix(cpapr_ctx *ctx, const void *src, int64_t rows, double *dst) {
     const int R = ctx->R, Rp = ctx->Rp;
     const int64_t n = rows * Rp;
-    const double *from = (const double *)src;
-    if (ctx->esize != 8) {
-        widen_kernel<float><<<grid_for(n), 256, 0, ctx->stream>>>((const float *)src, ctx->stage, n);
-        count_launch(ctx);
-        CPAPR_CUDA(ctx, cudaGetLastError());
-        from = ctx->stage;
-    }
-    if (rows > 0)
-        CPAPR_CUDA(ctx, cudaMemcpy2DAsync(dst, (size_t)R * 8, from, (size_t)Rp * 8, (size_t)R * 8, (size_t)rows,
+    if (rows <= 0) return CPAPR_OK;
+    if (ctx->esize == 8) {
+        CPAPR_CUDA(ctx, cudaMemcpy2DAsync(dst, (size_t)R * 8, src, (size_t)Rp * 8, (size_t)R * 8, (size_t)rows,
                                           cudaMemcpyDefault, ctx->stream));
+        return CPAPR_OK;
+    }
+    // FP32: widened and packed at once, straight into the caller's device memory
+    // where the kernel can write it
+    int lg = 0;
+    while ((1 << lg) < Rp) ++lg;
+    const bool dev = device_doubles(ctx, dst);
+    widen_kernel<float><<<grid_for(n), 256, 0, ctx->stream>>>((const float *)src, dev ? dst : ctx->stage, n, R, lg);
+    count_launch(ctx);
+    CPAPR_CUDA(ctx, cudaGetLastError());
+    if (!dev)
+        CPAPR_CUDA(ctx, cudaMemcpyAsync(dst, ctx->stage, (size_t)rows * R * 8, cudaMemcpyDefault, ctx->stream));
     return CPAPR_OK;
 }
 

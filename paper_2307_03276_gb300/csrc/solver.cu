@@ -107,21 +107,16 @@ static cpapr_status enqueue_mode(cpapr_ctx *ctx, int n, double tol, int max_inne
     return CPAPR_OK;
 }
 
-// Enqueues the log-likelihood of the current model and its copy to *host
-// (complete after the context's stream is synchronised).
-cpapr_status loglik_enqueue(cpapr_ctx *ctx, double *host) {
-    CPAPR_TRY(launch_loglik(ctx, ctx->scalars));
-    CPAPR_CUDA(ctx, cudaMemcpyAsync(host, ctx->scalars, 8, cudaMemcpyDeviceToHost, ctx->stream));
-    return CPAPR_OK;
-}
-
+// The log-likelihood of the current model, and with it the flag of the bounded
+// waits (errflag[3], left in ctx->host for the caller's check).
 static cpapr_status loglik_now(cpapr_ctx *ctx, double *host) {
-    CPAPR_TRY(loglik_enqueue(ctx, host));
+    CPAPR_TRY(launch_loglik(ctx, ctx->scalars));
+    CPAPR_CUDA(ctx, cudaMemcpyAsync(&ctx->host->ll, ctx->scalars, 8, cudaMemcpyDeviceToHost, ctx->stream));
+    CPAPR_CUDA(ctx, cudaMemcpyAsync(&ctx->host->flags[3], ctx->errflag + 3, 4, cudaMemcpyDeviceToHost, ctx->stream));
     CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    *host = ctx->host->ll;
     return CPAPR_OK;
 }
-
-cpapr_status launch_loglik_host(cpapr_ctx *ctx, double *host) { return loglik_now(ctx, host); }
 
 cpapr_status batch_mu_solve_persistent(cpapr_ctx *const *ctxs, int count, double tol, int max_outer, int max_inner,
                                        cpapr_result *results);
@@ -129,14 +124,14 @@ cpapr_status batch_mu_solve_persistent(cpapr_ctx *const *ctxs, int count, double
 cpapr_status mu_solve(cpapr_ctx *ctx, double tol, int max_outer, int max_inner, cpapr_result *res,
                       int32_t *inner_trace, double *ll_trace, double *kkt_trace) {
     const int N = ctx->N;
-    std::vector<InnerState> hs(N);
+    const InnerState *hs = ctx->host->inner;
     int outer = 0, total_inner = 0;
     bool conv = false;
     double kkt_last = 0.0;
     for (int k = 0; k < max_outer; ++k) {
         const bool shift = ctx->k_total > 0;
         for (int n = 0; n < N; ++n) CPAPR_TRY(enqueue_mode(ctx, n, tol, max_inner, shift));
-        CPAPR_CUDA(ctx, cudaMemcpyAsync(hs.data(), ctx->inner, sizeof(InnerState) * N, cudaMemcpyDeviceToHost,
+        CPAPR_CUDA(ctx, cudaMemcpyAsync(ctx->host->inner, ctx->inner, sizeof(InnerState) * N, cudaMemcpyDeviceToHost,
                                         ctx->stream));
         CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
         ctx->k_total += 1;
