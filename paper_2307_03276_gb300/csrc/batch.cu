@@ -61,9 +61,9 @@ struct BatchCtl {
 };
 
 // rank classes of the batched Phi kernel: (ranks per lane, lanes), ranks up
-// to 32.  All classes are inlined into one kernel, so its registers are the
-// largest class's: FP32 keeps one float4 per lane; FP64 one lane up to 8
-// ranks and lanes of 8 ranks above (the single-tensor heuristic's choices).
+// to 32.  All classes are in one kernel, so its registers are the largest
+// class's: FP32 keeps one float4 per lane; FP64 one lane up to 8 ranks and lanes
+// of 8 ranks above (the single-tensor heuristic's choices).
 template <typename T> struct Classes;
 template <> struct Classes<float> {
     static constexpr int n = 4;
@@ -94,11 +94,14 @@ template <typename T, int OP> __host__ __device__ constexpr bool batch_direct() 
 template <typename T, int OP> __host__ __device__ constexpr int batch_block() {
     return batch_direct<T, OP>() ? kDirectThreads : batch_threads<T>();
 }
-// resident blocks per SM the registers are held to (measured on GB300): the
-// FP32 classes all keep one float4 per lane, like the single-tensor kernel's
-// four-block case; every FP64 class fits three blocks (168 registers)
+// resident blocks per SM the registers are held to (measured on GB300).  The Phi
+// kernels call each rank class as a function (direct_class, staged_class), so a
+// launch is not held to the registers of all classes inlined side by side with a
+// copy of the tensor's arguments (FP64: 168 and three blocks, 74.1 ms for two outer
+// iterations of the 64 tensors; as functions 128 and four blocks, 72.4; five 73.5);
+// the log-likelihood keeps its classes inline.
 template <typename T, int OP = OP_LL> __host__ __device__ constexpr int batch_min_blocks() {
-    return batch_direct<T, OP>() ? 6 : sizeof(T) == 8 ? 3 : 4;
+    return batch_direct<T, OP>() ? 6 : sizeof(T) == 8 ? (OP == OP_PHI ? 4 : 3) : 4;
 }
 
 // One class's direct tile as a function of its own: four of them inlined side by
@@ -106,6 +109,12 @@ template <typename T, int OP = OP_LL> __host__ __device__ constexpr int batch_mi
 template <int NM1, int G, int OP, bool PI>
 __device__ __noinline__ void direct_class(const PhiArgs &a, int tile, unsigned char *smem, double *red) {
     direct_tile<NM1, G, OP, PI>(a, tile, smem, red);
+}
+
+template <typename T, int NM1, int RPL, int G, int U, bool PI>
+__device__ __noinline__ bool staged_class(const PhiArgs &a, int tile, unsigned char *smem, double *red, uint64_t *bar,
+                                          uint32_t &phase) {
+    return phi_tile_body<T, NM1, RPL, G, OP_PHI, batch_threads<T>(), U, PI>(a, tile, smem, red, bar, phase);
 }
 
 template <typename T, int NM1, int K, int OP, bool PI = false>
@@ -116,6 +125,8 @@ __device__ __forceinline__ bool run_class(const PhiArgs &a, int tile, unsigned c
     if constexpr (batch_direct<T, OP>()) {
         direct_class<NM1, G, OP, PI>(a, tile, smem, red);
         return true;
+    } else if constexpr (OP == OP_PHI) {
+        return staged_class<T, NM1, RPL, G, batch_unroll<T, RPL, G>(), PI>(a, tile, smem, red, bar, phase);
     } else
         return phi_tile_body<T, NM1, RPL, G, OP, batch_threads<T>(), batch_unroll<T, RPL, G>(), PI>(a, tile, smem, red,
                                                                                                bar, phase);
@@ -158,7 +169,7 @@ __global__ void __launch_bounds__(batch_block<T, OP>(), batch_min_blocks<T, OP>(
         __syncthreads();
         if (it >= nitems) break;
         const int2 w = items[it];
-        if constexpr (batch_direct<T, OP>()) {
+        if constexpr (OP == OP_PHI) {
             // the tile reads its arguments from shared memory (the previous
             // item's last reads are behind the barriers above)
             __shared__ PhiArgs s_a;
@@ -166,17 +177,19 @@ __global__ void __launch_bounds__(batch_block<T, OP>(), batch_min_blocks<T, OP>(
             for (int k = threadIdx.x; k < (int)(sizeof(PhiArgs) / 4); k += batch_block<T, OP>())
                 reinterpret_cast<uint32_t *>(&s_a)[k] = reinterpret_cast<const uint32_t *>(&desc[w.x].a)[k];
             __syncthreads();
-            if (!s_a.inner->done) run_item<T, NM1, OP, false>(s_a, desc[w.x].cfg, w.y, smem_raw, red, &bar, phase);
-            continue;
-        }
-        const PhiArgs a = desc[w.x].a;
-        if constexpr (sizeof(T) == 8 && OP == OP_PHI) {
-            if (a.pi) {
-                ok = run_item<T, NM1, OP, true>(a, desc[w.x].cfg, w.y, smem_raw, red, &bar, phase);
-                continue;
+            if (s_a.inner->done) continue;
+            const int cfg = desc[w.x].cfg;
+            if constexpr (sizeof(T) == 8) {
+                if (s_a.pi) {
+                    ok = run_item<T, NM1, OP, true>(s_a, cfg, w.y, smem_raw, red, &bar, phase);
+                    continue;
+                }
             }
+            ok = run_item<T, NM1, OP, false>(s_a, cfg, w.y, smem_raw, red, &bar, phase);
+        } else {
+            const PhiArgs a = desc[w.x].a;
+            ok = run_item<T, NM1, OP, false>(a, desc[w.x].cfg, w.y, smem_raw, red, &bar, phase);
         }
-        ok = run_item<T, NM1, OP, false>(a, desc[w.x].cfg, w.y, smem_raw, red, &bar, phase);
     }
     // the last block out resets the work counter for the next launch
     if (threadIdx.x == 0) {
@@ -448,7 +461,8 @@ struct ModePlan {
     int ntiles = 0, nchunks = 0, nechunks = 0;
     cudaGraphExec_t exec = nullptr;
     int body_kernels = 0;
-    size_t smem = 0;  // dynamic shared memory of the Phi launch (largest tile of the batch)
+    size_t smem = 0;      // dynamic shared memory of the log-likelihood launch (largest tile of the batch)
+    size_t smem_phi = 0;  // and of the Phi launches, which stage no coordinates where the rows are materialised
     int2 *pitems = nullptr;  // (tensor, chunk) items of the batched Khatri-Rao row build
     int npitems = 0;
 };
@@ -483,7 +497,7 @@ Plan *g_cache = nullptr;
 
 template <typename T>
 cudaError_t launch_phi_batch(const ModePlan &mp, int nm1, int grid, BatchCtl *ctl, cudaStream_t s) {
-    const size_t smem = batch_direct<T, OP_PHI>() ? direct_smem() : mp.smem;
+    const size_t smem = batch_direct<T, OP_PHI>() ? direct_smem() : mp.smem_phi;
     auto go = [&](auto kern) {
         if (smem > 48 * 1024) cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         kern<<<grid, batch_block<T, OP_PHI>(), smem, s>>>(mp.desc, mp.tiles, mp.ntiles, ctl);
@@ -706,7 +720,7 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
             for (int n = 0; n < N; ++n) sp[(size_t)i * N + n] = ctxs[i]->inner + n;
         BT_CUDA(cudaMemcpy(P.state_ptrs, sp.data(), sp.size() * sizeof(InnerState *), cudaMemcpyHostToDevice));
     }
-    size_t smem_max = 0;
+    size_t smem_max = 0, smem_phi = 0;
     std::vector<BatchTensor> desc0;
     for (int n = 0; n < N; ++n) {
         ModePlan &mp = P.modes[n];
@@ -783,10 +797,14 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
         });
         mp.ntiles = (int)tiles.size();
         {
-            int maxtile = 4;
-            for (int i = 0; i < count; ++i) maxtile = std::max(maxtile, desc[i].a.T);
-            mp.smem = phi_smem_bytes(maxtile, N - 1, (int)sizeof(T), batch_threads<T>(), maxrpl);
-            smem_max = std::max(smem_max, mp.smem);
+            for (int i = 0; i < count; ++i) {
+                const PhiArgs &ai = desc[i].a;
+                const size_t all = phi_smem_bytes(std::max(4, ai.T), N - 1, (int)sizeof(T), batch_threads<T>(), maxrpl);
+                smem_max = std::max(smem_max, all);
+                smem_phi = std::max(smem_phi, ai.pi ? phi_smem_bytes(std::max(4, ai.T), 0, (int)sizeof(T),
+                                                                     batch_threads<T>(), maxrpl)
+                                                    : all);
+            }
         }
         mp.nchunks = (int)chunks.size();
         mp.nechunks = (int)echunks.size();
@@ -828,8 +846,11 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
         drop_cache_locked();
         return fail(c0, CPAPR_E_ARG, "batch: tile_nnz too large for the shared-memory stage");
     }
-    for (int n = 0; n < N; ++n) P.modes[n].smem = smem_max;  // one occupancy for the whole plan
-    P.grid = persistent_grid<T>(N - 1, smem_max);
+    for (int n = 0; n < N; ++n) {  // one occupancy for the whole plan
+        P.modes[n].smem = smem_max;
+        P.modes[n].smem_phi = smem_phi;
+    }
+    P.grid = persistent_grid<T>(N - 1, smem_phi);
     if (graph_flag)
         for (int n = 0; n < N; ++n) {
             cpapr_status st = build_graph<T>(c0, P, n, tol, max_inner, P.grid);
