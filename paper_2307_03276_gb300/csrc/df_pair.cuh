@@ -16,6 +16,10 @@
 // n are then scaled by 2^K, K = (N - 1) c - sum_{m != n} k_m, and are at most about
 // 2^(kPairTop + N - 1).  Pairs hold scaled values in [2^kPairLow, 2^(e_max + 1)).
 //
+// Layout.  A row holds its columns two by two: hi of column 2v and of 2v + 1, then
+// their lo parts, 16 bytes; so a load brings both parts of two columns as the
+// operands of packed FP32 instructions.
+//
 // Error.  A factor pair is rounded to 2^-49 relative at most; a product
 // (pair_mul: one exact FP32 product, the two cross products, renormalised)
 // adds at most 2^-47, about 1e-15 in the mean.
@@ -43,6 +47,12 @@ __device__ __forceinline__ double escape_value(float2 p) {
     const unsigned long long b =
         ((unsigned long long)(__float_as_uint(p.x) & 0x7fffffffu) << 32) | __float_as_uint(p.y);
     return __longlong_as_double((long long)b);
+}
+
+// column c of the row of pairs that starts `row` columns into `base`
+__device__ __forceinline__ float2 pair_at(const float *base, int64_t row, int c) {
+    const float *p = base + 2 * row + 4 * (c >> 1) + (c & 1);
+    return make_float2(__ldg(p), __ldg(p + 2));
 }
 
 // v 2^s as a pair, or v as an escape where v 2^s lies outside [2^kPairLow, 2^(emax + 1))

@@ -7,12 +7,13 @@
 // element) and issued one DFMA per element for the scale-add, 64 cycles of an
 // SM quarter's FP64 pipe per warp instruction: 63 issue slots and 64 FP64 cycles
 // per element.  Now the pairs are built once per mode and outer iteration and an
-// element costs about 18 FP32 operations and no FP64 one (the FP32 sums move to
-// an FP64 accumulator every 16 nonzeros).  A launch on the 4-way tensor with 5e7
-// nonzeros (R = 16) went from 2.67 to 1.37 ms (0.70 of the HBM peak for its 6.45 GB),
-// on the 3-way one with 1e7 (R = 32) from 0.95 to 0.61 ms; what bounds it now is
-// instruction issue (about 55% of the slots, the rest waits for loads and for
-// the block's slowest warp at a tile's end).
+// element costs about 18 FP32 operations, two columns per packed instruction, and
+// no FP64 one (the FP32 sums move to an FP64 accumulator every 16 nonzeros).  A
+// launch on the 4-way tensor with 5e7 nonzeros (R = 16) went from 2.67 to 1.31 ms
+// (0.73 of the HBM peak for its 6.45 GB), on the 3-way one with 1e7 (R = 32) from
+// 0.95 to 0.58 ms (0.68); 1.37 and 0.61 before the packed instructions.  What bounds
+// it now is instruction issue and the waits that too few warps (20 per SM) leave
+// open: loads of the next step, and the block's slowest warp at a tile's end.
 //
 // Scaled quantities (all powers of two): pi' = pi 2^K (the pairs), b' = b 2^(S - K),
 // eps' = eps 2^S, s' = s 2^S with S = kDfS; v' = v 2^V with V = kDfV; sums of
@@ -44,9 +45,9 @@ namespace cpapr {
 constexpr int kDfS = 60;
 constexpr int kDfV = 10;
 constexpr int kDfThreads = 128;
-// Resident blocks per SM the registers are held to (96 each).  With six (80 and
-// more spills) a launch took 1.45 against 1.37 ms (4-way, 5e7 nonzeros, R = 16) and
-// 0.62 against 0.61 ms (3-way, 1e7, R = 32); with four 1.44 and 0.78.
+// Resident blocks per SM the registers are held to (96 each).  4 / 5 / 6 blocks:
+// 1.43 / 1.31 / 1.36 ms a launch (4-way, 5e7 nonzeros, R = 16), 0.64 / 0.58 / 0.59 ms
+// (3-way, 1e7, R = 32); six (80 registers) spill.
 constexpr int kDfBlocks = 5;
 constexpr int kDfSpill = 16;  // nonzeros summed in FP32 pairs before they move to FP64
 
@@ -86,33 +87,42 @@ __device__ __forceinline__ float2 df_add(float2 a, float2 b) {
     return make_float2(h, e - (h - s));
 }
 
-// S + C += a b for pairs a, b >= 0.  t = S + a_hi b_hi is rounded once (FMA); its
-// error is (S - (t - z)) + (a_hi b_hi - z) with z = t - S as in Knuth's two-sum: the
-// first part is exact, the second is an FMA whose rounding is 2^-24 of it, 2^-48 of
-// t.  The error and the cross terms go to C: nine operations (twelve with the
-// product and the sum taken apart).
-__device__ __forceinline__ void df_fma(float ah, float al, float2 b, float &S, float &C) {
-    const float t = fmaf(ah, b.x, S);
-    const float z = t - S;
-    const float d = S - (t - z);
-    const float r = fmaf(ah, b.x, -z);
-    C = fmaf(ah, b.y, C);
-    C = fmaf(al, b.x, C);
-    C += d + r;
+// S + C += a b for pairs a, b >= 0, two columns at once (.x and .y: Blackwell's
+// packed FP32 instructions take two per lane and issue slot; the kernel is bound by
+// issue).  t = S + a_hi b_hi is rounded once (FMA); its error is (S - (t - z)) +
+// (a_hi b_hi - z) with z = t - S as in Knuth's two-sum: the first part is exact, the
+// second is an FMA whose rounding is 2^-24 of it, 2^-48 of t.  The error and the
+// cross terms go to C: nine operations (twelve with the product and the sum
+// taken apart).  Differences are FMAs with -1, which round the same.
+__device__ __forceinline__ void df_fma2(float2 ah, float2 al, float2 bh, float2 bl, float2 &S, float2 &C) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 t = __ffma2_rn(ah, bh, S);
+    const float2 nz = __ffma2_rn(t, m1, S);                       // -z
+    const float2 e = __ffma2_rn(__fadd2_rn(t, nz), m1, S);        // S - (t - z)
+    const float2 r = __ffma2_rn(ah, bh, nz);
+    C = __ffma2_rn(ah, bl, C);
+    C = __ffma2_rn(al, bh, C);
+    C = __fadd2_rn(C, __fadd2_rn(e, r));
     S = t;
 }
 
-// <a, b> of two rows of pairs as a renormalised pair
-template <int K>
-__device__ __forceinline__ float2 df_dot(const float (&ah)[K], const float (&al)[K], const float2 (&b)[K]) {
-    float S = __fmul_rn(ah[0], b[0].x);  // not to be fused into the sums that follow
-    float C = fmaf(ah[0], b[0].x, -S);
-    C = fmaf(ah[0], b[0].y, C);
-    C = fmaf(al[0], b[0].x, C);
+// <a, b> of two rows of pairs as a renormalised pair: even and odd columns
+// side by side, then their sums added (two-sum)
+template <int VP>
+__device__ __forceinline__ float2 df_dot(const float2 (&ah)[VP], const float2 (&al)[VP], const float2 (&bh)[VP],
+                                         const float2 (&bl)[VP]) {
+    const float2 m1 = make_float2(-1.f, -1.f), zero = make_float2(0.f, 0.f);
+    float2 S = __fmul2_rn(ah[0], bh[0]);
+    float2 C = __ffma2_rn(ah[0], bh[0], __ffma2_rn(S, m1, zero));
+    C = __ffma2_rn(ah[0], bl[0], C);
+    C = __ffma2_rn(al[0], bh[0], C);
 #pragma unroll
-    for (int r = 1; r < K; ++r) df_fma(ah[r], al[r], b[r], S, C);
-    const float h = S + C;
-    return make_float2(h, C - (h - S));
+    for (int v = 1; v < VP; ++v) df_fma2(ah[v], al[v], bh[v], bl[v], S, C);
+    const float t = S.x + S.y;
+    const float z = t - S.x;
+    const float c = ((S.x - (t - z)) + (S.y - z)) + (C.x + C.y);
+    const float h = t + c;
+    return make_float2(h, c - (h - t));
 }
 
 // (xh + xl) / max(s, eps) as a pair: q0 from the hardware reciprocal refined by
@@ -184,12 +194,12 @@ __device__ __forceinline__ float2 pair_exact(const PhiArgs &a, int nm1, int K, i
 template <bool PI>
 __device__ __forceinline__ float2 pair_reload(const PhiArgs &a, int nm1, int K, int p, int c) {
     if constexpr (PI) {
-        return __ldg(reinterpret_cast<const float2 *>(a.pi) + (int64_t)p * a.Rp + c);
+        return pair_at(reinterpret_cast<const float *>(a.pi), (int64_t)p * a.Rp, c);
     } else {
         PairProduct y;
 #pragma unroll 1
         for (int k = 0; k < nm1; ++k) {
-            const float2 f = __ldg(a.P[k] + (int64_t)__ldg(a.idx[k] + p) * a.Rp + c);
+            const float2 f = pair_at(reinterpret_cast<const float *>(a.P[k]), (int64_t)__ldg(a.idx[k] + p) * a.Rp, c);
             if (k == 0)
                 y.start(f);
             else
@@ -339,16 +349,16 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
         kkt = __longlong_as_double((long long)*((volatile unsigned long long *)&a.inner->kkt[l & 1]));
     }
 
-    float S[RPL], C[RPL], bh[RPL], bl[RPL];
+    float2 S[VP], C[VP], bh[VP], bl[VP];  // columns 2v (.x) and 2v + 1 (.y)
     float top = 0.f;  // largest b_hi of the lane's columns
     auto load_b = [&](int32_t row) {
         top = 0.f;
 #pragma unroll
         for (int v = 0; v < VP; ++v) {
             const double2 b = __ldg(reinterpret_cast<const double2 *>(Bm + (int64_t)row * Rp + col(v)));
-            df_cut(b.x, kDfS - K, bh[2 * v], bl[2 * v]);
-            df_cut(b.y, kDfS - K, bh[2 * v + 1], bl[2 * v + 1]);
-            top = fmaxf(top, fmaxf(bh[2 * v], bh[2 * v + 1]));
+            df_cut(b.x, kDfS - K, bh[v].x, bl[v].x);
+            df_cut(b.y, kDfS - K, bh[v].y, bl[v].y);
+            top = fmaxf(top, fmaxf(bh[v].x, bh[v].y));
         }
     };
     load_b(cur);
@@ -359,7 +369,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
 #pragma unroll
         for (int v = 0; v < VP; ++v) acc[v * G + lane] = make_double2(0.0, 0.0);
 #pragma unroll
-        for (int r = 0; r < RPL; ++r) S[r] = C[r] = 0.f;
+        for (int v = 0; v < VP; ++v) S[v] = C[v] = make_float2(0.f, 0.f);
     }
     int q = qa;
     // escapes left out of the current sums: the columns that had them (low 8 bits)
@@ -375,10 +385,10 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
 #pragma unroll
         for (int k = 0; k < VP; ++k) {
             const double2 t = acc[k * G + lane];
-            v[2 * k] = t.x + (df_widen(S[2 * k]) + df_widen(C[2 * k]));
-            v[2 * k + 1] = t.y + (df_widen(S[2 * k + 1]) + df_widen(C[2 * k + 1]));
+            v[2 * k] = t.x + (df_widen(S[k].x) + df_widen(C[k].x));
+            v[2 * k + 1] = t.y + (df_widen(S[k].y) + df_widen(C[k].y));
             acc[k * G + lane] = make_double2(0.0, 0.0);
-            S[2 * k] = C[2 * k] = S[2 * k + 1] = C[2 * k + 1] = 0.f;
+            S[k] = C[k] = make_float2(0.f, 0.f);
         }
         // escaped elements were left out: below 2^-80 of their v' in all, nothing in FP64
         // beside a sum of 2^-25 of them or more; a column with less is summed again
@@ -407,9 +417,11 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
                 const float kf = float_below(kkt);
                 const double *b = Bm + (int64_t)cur * Rp;
 #pragma unroll
-                for (int r = 0; r < RPL; ++r)
-                    if (!b_in_regs || !(bh[r] < 0x1p100f) || kkt_candidate(bh[r] * b_scale, v[r], kf))
+                for (int r = 0; r < RPL; ++r) {
+                    const float br = r % 2 ? bh[r / 2].y : bh[r / 2].x;
+                    if (!b_in_regs || !(br < 0x1p100f) || kkt_candidate(br * b_scale, v[r], kf))
                         kkt = tmax(kkt, viol_t(__ldg(b + col(r / 2) + r % 2), v[r]));
+                }
             }
         } else if (a.atomic) {
 #pragma unroll
@@ -424,7 +436,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
         }
     };
 
-    float2 pi[U][RPL];  // rows of the step at position q
+    float2 ph[U][VP], pl[U][VP];  // rows of the step at position q: hi and lo parts, columns as above
     // what a step reads: the materialised rows, or the coordinates of the rows to
     // form; its row starts; its counts
     int32_t ii[U][MAXK];
@@ -447,8 +459,8 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
 #pragma unroll
                 for (int v = 0; v < VP; ++v) {
                     const float4 y = __ldcs(P + v * G + lane);
-                    pi[u][2 * v] = make_float2(y.x, y.y);
-                    pi[u][2 * v + 1] = make_float2(y.z, y.w);
+                    ph[u][v] = make_float2(y.x, y.y);
+                    pl[u][v] = make_float2(y.z, y.w);
                 }
             } else {
 #pragma unroll
@@ -470,23 +482,29 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
                         const float4 y =
                             __ldg(reinterpret_cast<const float4 *>(a.P[k] + (int64_t)ii[u][k] * Rp) + v * G + lane);
                         if (k == 0) {
-                            y0.start(make_float2(y.x, y.y));
-                            y1.start(make_float2(y.z, y.w));
+                            y0.start(make_float2(y.x, y.z));
+                            y1.start(make_float2(y.y, y.w));
                         } else {
-                            y0.mul(make_float2(y.x, y.y));
-                            y1.mul(make_float2(y.z, y.w));
+                            y0.mul(make_float2(y.x, y.z));
+                            y1.mul(make_float2(y.y, y.w));
                         }
                     }
                 }
-                pi[u][2 * v] = y0.zero() ? make_float2(0.f, 0.f) : y0.p;
-                pi[u][2 * v + 1] = y1.zero() ? make_float2(0.f, 0.f) : y1.p;
+                const float2 e0 = y0.zero() ? make_float2(0.f, 0.f) : y0.p;
+                const float2 e1 = y1.zero() ? make_float2(0.f, 0.f) : y1.p;
+                ph[u][v] = make_float2(e0.x, e1.x);
+                pl[u][v] = make_float2(e0.y, e1.y);
                 bad |= (y0.pair_ok() || y0.zero() ? 0u : 1u) << (2 * v);
                 bad |= (y1.pair_ok() || y1.zero() ? 0u : 1u) << (2 * v + 1);
             }
             if (__builtin_expect(bad != 0u, 0)) {
 #pragma unroll
                 for (int r = 0; r < RPL; ++r)
-                    if ((bad >> r) & 1u) pi[u][r] = pair_exact(a, nm1, K, min(q + u, p1 - 1), col(r / 2) + r % 2);
+                    if ((bad >> r) & 1u) {
+                        const float2 e = pair_exact(a, nm1, K, min(q + u, p1 - 1), col(r / 2) + r % 2);
+                        (r % 2 ? ph[u][r / 2].y : ph[u][r / 2].x) = e.x;
+                        (r % 2 ? pl[u][r / 2].y : pl[u][r / 2].x) = e.y;
+                    }
             }
         }
     };
@@ -512,7 +530,8 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
 #pragma unroll
         for (int u = 0; u < U; ++u)
 #pragma unroll
-            for (int r = 0; r < RPL; ++r) top_bits = max(top_bits, __float_as_uint(pi[u][r].x));
+            for (int v = 0; v < VP; ++v)
+                top_bits = max(top_bits, max(__float_as_uint(ph[u][v].x), __float_as_uint(ph[u][v].y)));
         if (__builtin_expect((int)top_bits < 0, 0)) {
             // one above the pairs' window (beyond its factor's exponent), or any
             // where B is not safe, sends its nonzero to FP64
@@ -522,12 +541,15 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
             for (int u = 0; u < U; ++u) {
                 uint32_t e8 = 0, big = 0;
 #pragma unroll
-                for (int r = 0; r < RPL; ++r)
-                    if (is_escape(pi[u][r])) {
+                for (int r = 0; r < RPL; ++r) {
+                    float &h = r % 2 ? ph[u][r / 2].y : ph[u][r / 2].x;
+                    if ((int)__float_as_uint(h) < 0) {
                         e8 |= 1u << r;
-                        big = max(big, __float_as_uint(pi[u][r].x));
-                        pi[u][r] = make_float2(0.f, 0.f);
+                        big = max(big, __float_as_uint(h));
+                        h = 0.f;
+                        (r % 2 ? pl[u][r / 2].y : pl[u][r / 2].x) = 0.f;
                     }
+                }
                 if (u < m) {
                     em |= e8 << (8 * u);
                     if (e8 && (unsafe || big >= high)) redo |= 1u << u;
@@ -537,7 +559,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
 
         float2 s2[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) s2[u] = df_dot<RPL>(bh, bl, pi[u]);
+        for (int u = 0; u < U; ++u) s2[u] = df_dot<VP>(bh, bl, ph[u], pl[u]);
 
         float vh[U], vl[U];
         double m_ll = 1.0;
@@ -618,17 +640,19 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
                 }
             }
 #pragma unroll
-            for (int u = 0; u < U; ++u)
+            for (int u = 0; u < U; ++u) {
+                const float2 h2 = make_float2(vh[u], vh[u]), l2 = make_float2(vl[u], vl[u]);
 #pragma unroll
-                for (int r = 0; r < RPL; ++r) df_fma(vh[u], vl[u], pi[u][r], S[r], C[r]);
+                for (int v = 0; v < VP; ++v) df_fma2(h2, l2, ph[u][v], pl[u][v], S[v], C[v]);
+            }
             if (step % (kDfSpill / U) == 0) {
 #pragma unroll
                 for (int k = 0; k < VP; ++k) {
                     double2 t = acc[k * G + lane];
-                    t.x += df_widen(S[2 * k]) + df_widen(C[2 * k]);
-                    t.y += df_widen(S[2 * k + 1]) + df_widen(C[2 * k + 1]);
+                    t.x += df_widen(S[k].x) + df_widen(C[k].x);
+                    t.y += df_widen(S[k].y) + df_widen(C[k].y);
                     acc[k * G + lane] = t;
-                    S[2 * k] = C[2 * k] = S[2 * k + 1] = C[2 * k + 1] = 0.f;
+                    S[k] = C[k] = make_float2(0.f, 0.f);
                 }
             }
         }

@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(256) pair_factor_kernel(const double2 *__restr
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nv; e += (int64_t)gridDim.x * blockDim.x) {
         const double2 x = A[e];
         const float2 p = pair_encode(x.x, c - k, c), q = pair_encode(x.y, c - k, c);
-        P[e] = make_float4(p.x, p.y, q.x, q.y);
+        P[e] = make_float4(p.x, q.x, p.y, q.y);
     }
 }
 
@@ -65,11 +65,11 @@ __global__ void __launch_bounds__(256) pi_pair_kernel(const PhiArgs a, float4 *_
                 ii[k] = __ldg(a.idx[k] + p);
                 const float4 x = __ldg(reinterpret_cast<const float4 *>(a.P[k] + (int64_t)ii[k] * a.Rp) + v);
                 if (k == 0) {
-                    q0.start(make_float2(x.x, x.y));
-                    q1.start(make_float2(x.z, x.w));
+                    q0.start(make_float2(x.x, x.z));
+                    q1.start(make_float2(x.y, x.w));
                 } else {
-                    q0.mul(make_float2(x.x, x.y));
-                    q1.mul(make_float2(x.z, x.w));
+                    q0.mul(make_float2(x.x, x.z));
+                    q1.mul(make_float2(x.y, x.w));
                 }
             }
         }
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(256) pi_pair_kernel(const PhiArgs a, float4 *_
         };
         if (!q0.pair_ok()) q0.p = q0.zero() ? make_float2(0.f, 0.f) : exact(2 * v);
         if (!q1.pair_ok()) q1.p = q1.zero() ? make_float2(0.f, 0.f) : exact(2 * v + 1);
-        __stcs(pi + e, make_float4(q0.p.x, q0.p.y, q1.p.x, q1.p.y));
+        __stcs(pi + e, make_float4(q0.p.x, q1.p.x, q0.p.y, q1.p.y));
     }
 }
 
