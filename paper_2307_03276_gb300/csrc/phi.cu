@@ -108,6 +108,7 @@ uint32_t injected_stage_shortfall() {
 bool uses_pairs(const cpapr_ctx *ctx, int n) {
     const ModeLayout &L = ctx->mode[n];
     const int dot = ctx->opt.fp64_dot;
+    if (L.tile_nnz == 0) return false;  // not configured yet
     return ctx->esize == 8 && ctx->nnz > 0 && ctx->Rp / L.lanes <= 8 && ctx->opt.eps >= 0x1p-43 &&
            ctx->opt.eps <= 0x1p20 &&
            (dot == CPAPR_DOT_FP32_PIPE ||
