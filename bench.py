@@ -72,19 +72,22 @@ NCU_TRAFFIC = {
     ("c2_3way_1e5x1e5x1e3_1e7_r32", "f64", "materialised", (4, 4, 4), (1024, 1024, 1024)):
         {"bytes": [2668266240 + 18964736, 2667915520 + 16923904, 2642699520 + 6055680], "nnz": 10_000_000,
          "source": "ncu capture of the FP64 materialised-Pi tile kernel, modes 0-2"},
+    ("c2_3way_1e5x1e5x1e3_1e7_r32", "f64", "materialised", (4, 4, 4), (2048, 2048, 2048)):
+        {"bytes": [2754560256 + 18587648, 2754175744 + 13909760, 2717311488 + 2564608], "nnz": 10_000_000,
+         "source": "ncu capture of the FP64 kernel over float-pair rows, modes 0-2"},
     ("c2_3way_1e5x1e5x1e3_1e7_r32", "f32", "fused", (8, 8, 8), (2048, 2048, 2048)):
-        {"bytes": [149920512 + 9855744, 149870848 + 6829568, 150985472 + 916480], "nnz": 10_000_000,
-         "l2_read": [46078048 * 32, 45825406 * 32, 56520460 * 32],
-         "source": "ncu capture of the FP32 fused-Pi tile kernel, modes 0-2"},
-    ("c3_4way_2e5x2e5x1e4x365_5e7_r16", "f64", "materialised", (2, 2, 2, 2), (2048, 2048, 2048, 2048)):
-        {"bytes": [1386862336 + 12523776, 1386850048 + 12308224, 1362785024 + 3010048, 1361540096 + 3038976],
+        {"bytes": [150362368 + 10147072, 150232320 + 6955776, 152147968 + 890880], "nnz": 10_000_000,
+         "l2_read": [41971897 * 32, 41853581 * 32, 51656501 * 32],
+         "source": "ncu capture of the FP32 direct kernel, fused Pi, modes 0-2"},
+    ("c3_4way_2e5x2e5x1e4x365_5e7_r16", "f64", "materialised", (2, 2, 2, 2), (4096, 4096, 4096, 4096)):
+        {"bytes": [1449559040 + 13676288, 1444822272 + 11705344, 1403012352 + 1873664, 1400862464 + 2439424],
          "nnz": 10_000_000,
-         "source": "ncu capture of the FP64 materialised-Pi tile kernel, modes 0-3, on the 4-way tensor's "
+         "source": "ncu capture of the FP64 kernel over float-pair rows, modes 0-3, on the 4-way tensor's "
                    "1e7-nonzero copy (same dims), scaled to 5e7 nonzeros"},
     ("c3_4way_2e5x2e5x1e4x365_5e7_r16", "f32", "materialised", (4, 4, 4, 4), (4096, 4096, 4096, 4096)):
-        {"bytes": [694905088 + 3333888, 694989056 + 212992, 682062336 + 261888, 681425920 + 171520],
+        {"bytes": [714250752 + 3482112, 714228992 + 947968, 701437952 + 862720, 700708864 + 556288],
          "nnz": 10_000_000,
-         "source": "ncu capture of the FP32 materialised-Pi tile kernel, modes 0-3, on the 4-way tensor's "
+         "source": "ncu capture of the FP32 direct kernel, materialised Pi, modes 0-3, on the 4-way tensor's "
                    "1e7-nonzero copy (same dims), scaled to 5e7 nonzeros"},
 }
 
@@ -585,9 +588,19 @@ def ncu_traffic(T, dtype, mat, info, inner_per_mode):
     return sum(w[n] * per_mode[n] for n in range(N)) / tot, ent["source"], l2
 
 
-def roofline_for(T, inner_per_mode, stats, precision, peaks, cp, pi_modes=None, info=None):
+def on_pairs(T, info) -> bool:
+    """Whether the FP64 Phi launches run on float pairs (the library's automatic
+    choice): 8 or fewer ranks per lane and at least 608 tiles of 2048 nonzeros
+    (1024 from rank 17 on)."""
+    rp = info.rank_padded
+    tile = 2048 if rp <= 16 else 1024
+    return rp // max(int(info.rank_lanes[0]), 1) <= 8 and -(-T.nnz // tile) >= 608
+
+
+def roofline_for(T, inner_per_mode, stats, precision, peaks, cp, pi_modes=None, info=None, pairs=False):
     """Roofline of the Phi tile kernel from its measured average duration.
-    pi_modes: per mode, whether Phi streamed materialised Khatri-Rao rows."""
+    pi_modes: per mode, whether Phi streamed materialised Khatri-Rao rows.
+    pairs: FP64 on float-pair rows, no FP64 arithmetic per element: HBM is the bound."""
     N, nnz, R = T.nmodes, T.nnz, T.rank
     fb = 8 if precision == cp.CPAPR_FP64 else 4
     mat = [bool(pi_modes and pi_modes[n] == cp.CPAPR_PI_MATERIALISED) for n in range(N)]
@@ -615,7 +628,13 @@ def roofline_for(T, inner_per_mode, stats, precision, peaks, cp, pi_modes=None, 
             l2g["l2_served"] = l2_read / (total_ms / max(launches, 1) / 1e3) / 1e9
             l2g["frac"] = l2g["l2_served"] / L2_GATHER_GBS
     form = "materialised Pi" if all(mat) else ("fused Pi" if not any(mat) else "mixed")
-    if precision == cp.CPAPR_FP64:
+    if precision == cp.CPAPR_FP64 and pairs:
+        roof = {"bound": "hbm", "achieved": hbm["achieved"], "peak": hbm["peak"], "unit": "GB/s",
+                "frac": hbm["frac"], "traffic": traffic, "kernel": f"phi_pair_kernel ({form})",
+                "peak_source": f"{peaks['source']} hbm_gbs",
+                "paper_flop_model": {"achieved": fl / sec / 1e12, "unit": "TFLOP/s",
+                                     "per_nonzero": "4R+2" if all(mat) else "(N+2)R+2"}}
+    elif precision == cp.CPAPR_FP64:
         ach = fl64 / sec / 1e12
         dot32 = all(on32)
         model = ("2R" if all(mat) else "NR") if dot32 else ("4R+2" if all(mat) else "(N+2)R+2")
@@ -629,7 +648,7 @@ def roofline_for(T, inner_per_mode, stats, precision, peaks, cp, pi_modes=None, 
                                      "per_nonzero": "4R+2" if all(mat) else "(N+2)R+2"}}
     else:
         roof = {"bound": "hbm", "achieved": hbm["achieved"], "peak": hbm["peak"], "unit": "GB/s",
-                "frac": hbm["frac"], "traffic": traffic, "kernel": f"phi_tile_kernel<float> ({form})",
+                "frac": hbm["frac"], "traffic": traffic, "kernel": f"direct_kernel ({form})",
                 "peak_source": f"{peaks['source']} hbm_gbs"}
     roof["traffic_unit"] = "bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)"
     roof["traffic_source"] = traffic_src
@@ -715,7 +734,7 @@ def run_ours(args):
     units = float(res["inner"].sum()) * T.nnz
     units_all, sec = aggregate(dist, units, res["ms"] / 1e3, use_cuda)
     roof = roofline_for(T, res["inner"], res["stats"], prim, peaks, cp, list(res["info"].pi_mode)[:T.nmodes],
-                        res["info"])
+                        res["info"], on_pairs(T, res["info"]))
     out = {"metric": METRIC, "value": units_all / sec, "unit": UNIT, "n_gpus": world, "steps": args.steps,
            "warmup": args.warmup, "ms_per_step": sec * 1e3 / args.steps, "higher_is_better": True,
            "scaling": "weak", "vs_baseline": None, "dtype": "f64" if prim == cp.CPAPR_FP64 else "f32",
@@ -739,7 +758,7 @@ def run_ours(args):
         out["variants"] = {name: {"value": u2 / s2, "unit": UNIT, "ms_per_step": s2 * 1e3 / args.steps,
                                   "dtype": "f32" if other == cp.CPAPR_FP32 else "f64",
                                   "roofline": roofline_for(T, r2["inner"], r2["stats"], other, peaks, cp,
-                                                           list(r2["info"].pi_mode)[:T.nmodes], r2["info"]),
+                                                           list(r2["info"].pi_mode)[:T.nmodes], r2["info"], on_pairs(T, r2["info"])),
                                   "inner_iterations_per_mode": r2["inner"].tolist(),
                                   "kernel_ms_per_step": kernel_breakdown(r2["stats"], args.steps),
                                   "loglik_last": r2["last"]["loglik"]}}
@@ -753,7 +772,7 @@ def run_ours(args):
             out["variants"]["fp64_fused_pi"] = {
                 "value": u3 / s3, "unit": UNIT, "ms_per_step": s3 * 1e3 / args.steps, "dtype": "f64",
                 "roofline": roofline_for(T, r3["inner"], r3["stats"], prim, peaks, cp,
-                                         list(r3["info"].pi_mode)[:T.nmodes], r3["info"]),
+                                         list(r3["info"].pi_mode)[:T.nmodes], r3["info"], on_pairs(T, r3["info"])),
                 "inner_iterations_per_mode": r3["inner"].tolist(),
                 "kernel_ms_per_step": kernel_breakdown(r3["stats"], args.steps),
                 "loglik_last": r3["last"]["loglik"]}
@@ -775,7 +794,7 @@ def run_ours(args):
                 c2[pname] = {"value": u4 / s4, "unit": UNIT, "steps": k2, "ms_per_step": s4 * 1e3 / k2,
                              "dtype": "f64" if prec == cp.CPAPR_FP64 else "f32",
                              "roofline": roofline_for(T2, r4["inner"], r4["stats"], prec, peaks, cp,
-                                                      list(r4["info"].pi_mode)[:T2.nmodes], r4["info"]),
+                                                      list(r4["info"].pi_mode)[:T2.nmodes], r4["info"], on_pairs(T2, r4["info"])),
                              "kernel_ms_per_step": kernel_breakdown(r4["stats"], k2)}
             out["variants"]["c2"] = c2
             del T2
@@ -904,8 +923,9 @@ def run_r_sweep(args):
                    "rank_lanes": list(info.rank_lanes)[:N], "tile_nnz": list(info.tile_nnz)[:N],
                    "reduction": list(info.reduction)[:N], "pi_mode": pim,
                    "phi_ms_per_launch": per, "phi_nnz_per_s": T.nnz / (per / 1e3),
-                   "phi_hbm_frac": byts / (per / 1e3) / 1e9 / peaks["hbm_gbs"],
-                   "phi_fp64_frac": (fl / (per / 1e3) / 1e12 / FP64_PEAK_TFLOPS) if fb == 8 else None,
+                   "phi_on_pairs": fb == 8 and on_pairs(T, info), "phi_hbm_frac": byts / (per / 1e3) / 1e9 / peaks["hbm_gbs"],
+                   "phi_fp64_frac": (fl / (per / 1e3) / 1e12 / FP64_PEAK_TFLOPS)
+                   if fb == 8 and not on_pairs(T, info) else None,
                    "pi_build_ms_per_launch": (bms / bl) if bl else None,
                    "mttkrp_ms_per_launch": mper, "mttkrp_nnz_per_s": T.nnz / (mper / 1e3),
                    "mttkrp_hbm_frac": mb / (mper / 1e3) / 1e9 / peaks["hbm_gbs"]}

@@ -76,6 +76,8 @@ enum { CPAPR_DOT_AUTO = 0, CPAPR_DOT_FP64 = 1, CPAPR_DOT_FP32_PIPE = 2 };
  *             streams fit in shared memory (about 220 KB per block, e.g. at
  *             most 8192 for a 3-way FP64 tensor); E_ARG otherwise.
  *  rank_lanes lanes that share one nonzero (1..32, power of two); 0 = automatic.
+ *             (The kernels that work on float pairs, and the FP32 ones that stage
+ *             nothing, keep 4 ranks per lane of their own.)
  *  use_graph  1 = run each mode's inner loop as a CUDA graph with a device-side
  *             early exit (default), 0 = plain stream launches.
  *  autotune   1 = time candidate (tile_nnz, rank_lanes, reduction, pi_mode)
