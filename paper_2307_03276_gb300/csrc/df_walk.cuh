@@ -190,48 +190,69 @@ __device__ __forceinline__ float2 pair_exact(const PhiArgs &a, int nm1, int K, i
     return pair_encode(d, K, kPairMax);
 }
 
-// element c of nonzero p's row again (the walk zeroes escapes in place), the same bits
-template <bool PI>
-__device__ __forceinline__ float2 pair_reload(const PhiArgs &a, int nm1, int K, int p, int c) {
-    if constexpr (PI) {
-        return pair_at(reinterpret_cast<const float *>(a.pi), (int64_t)p * a.Rp, c);
-    } else {
-        PairProduct y;
-#pragma unroll 1
-        for (int k = 0; k < nm1; ++k) {
-            const float2 f = pair_at(reinterpret_cast<const float *>(a.P[k]), (int64_t)__ldg(a.idx[k] + p) * a.Rp, c);
-            if (k == 0)
-                y.start(f);
-            else
-                y.mul(f);
-        }
-        return y.pair_ok() ? y.p : y.zero() ? make_float2(0.f, 0.f) : pair_exact(a, nm1, K, p, c);
-    }
-}
-
-// this lane's columns of nonzero p's row in FP64, and its part of <B[row], pi>
-template <int RPL, int G, bool PI>
+// this lane's columns of nonzero p's row in FP64, and its part of <B[row], pi>; a row
+// formed in place loads all its coordinates, then all its factor entries, at once
+template <int NM1, int RPL, int G, bool PI>
 __device__ __forceinline__ double pair_row64(const PhiArgs &a, int nm1, int K, int p, int row, int lane,
                                              double (&pv)[RPL]) {
     const double *B = reinterpret_cast<const double *>(a.B) + (int64_t)row * (RPL * G);
+    constexpr int Rp = RPL * G, MAXK = NM1 > 0 ? NM1 : kMaxNm1;
     double d = 0.0;
+    if constexpr (PI) {
 #pragma unroll
-    for (int r = 0; r < RPL; ++r) {
-        const int c = ((r >> 1) * G + lane) * 2 + (r & 1);
-        pv[r] = pair_value(pair_reload<PI>(a, nm1, K, p, c), K);
-        d = fma(__ldg(B + c), pv[r], d);
+        for (int r = 0; r < RPL; ++r)
+            pv[r] = pair_value(pair_at(reinterpret_cast<const float *>(a.pi), (int64_t)p * Rp, ((r >> 1) * G + lane) * 2 + (r & 1)), K);
+    } else {
+        int64_t at[MAXK];
+#pragma unroll
+        for (int k = 0; k < MAXK; ++k) at[k] = k < nm1 ? (int64_t)__ldg(a.idx[k] + p) * Rp : 0;
+#pragma unroll
+        for (int v = 0; v < RPL / 2; ++v) {
+            PairProduct<true> y0, y1;
+#pragma unroll
+            for (int k = 0; k < MAXK; ++k)
+                if (k < nm1) {
+                    const float4 y = __ldg(reinterpret_cast<const float4 *>(a.P[k] + at[k]) + v * G + lane);
+                    if (k == 0) {
+                        y0.start(make_float2(y.x, y.z));
+                        y1.start(make_float2(y.y, y.w));
+                    } else {
+                        y0.mul(make_float2(y.x, y.z));
+                        y1.mul(make_float2(y.y, y.w));
+                    }
+                }
+            if (y0.zero()) y0.p = make_float2(0.f, 0.f);
+            if (y1.zero()) y1.p = make_float2(0.f, 0.f);
+            const bool ok0 = y0.pair_ok() || y0.zero(), ok1 = y1.pair_ok() || y1.zero();
+            if (!(ok0 && ok1)) {
+                double2 f = make_double2(0.0, 0.0);
+#pragma unroll
+                for (int k = 0; k < MAXK; ++k)
+                    if (k < nm1) {
+                        const double2 g = __ldg(reinterpret_cast<const double2 *>(
+                                                    reinterpret_cast<const double *>(a.A[k]) + at[k]) + v * G + lane);
+                        f = k == 0 ? g : make_double2(f.x * g.x, f.y * g.y);
+                    }
+                if (!ok0) y0.p = pair_encode(f.x, K, kPairMax);
+                if (!ok1) y1.p = pair_encode(f.y, K, kPairMax);
+            }
+            pv[2 * v] = pair_value(y0.p, K);
+            pv[2 * v + 1] = pair_value(y1.p, K);
+        }
     }
+#pragma unroll
+    for (int r = 0; r < RPL; ++r) d = fma(__ldg(B + ((r >> 1) * G + lane) * 2 + (r & 1)), pv[r], d);
     return d;
 }
 
 // Nonzero p in FP64: a warp's lanes all call it, those of the groups that redo
 // their nonzero (`mine`) add v pi to their accumulators (Phi); returns x log m in
 // lane 0 of such a group (log-likelihood).
-template <int RPL, int G, int OP, bool PI>
+template <int NM1, int RPL, int G, int OP, bool PI>
 __device__ __forceinline__ double pair_redo(const PhiArgs &a, double2 *acc, int nm1, int K, int p, int row, int lane,
                                          bool mine) {
     double pv[RPL];
-    double d = pair_row64<RPL, G, PI>(a, nm1, K, p, row, lane, pv);
+    double d = pair_row64<NM1, RPL, G, PI>(a, nm1, K, p, row, lane, pv);
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
     if (!mine) return 0.0;
@@ -250,7 +271,7 @@ __device__ __forceinline__ double pair_redo(const PhiArgs &a, double2 *acc, int 
 
 // The columns `low` of v: the sums of v pi over one row's nonzeros from q - 1 back
 // to the row's start, or to qa, in FP64.  A group's lanes call it together.
-template <int RPL, int G, bool PI>
+template <int NM1, int RPL, int G, bool PI>
 __device__ __forceinline__ void pair_resum(const PhiArgs &a, int nm1, int K, int qa, int q, int row, int lane,
                                            unsigned gmask, uint32_t low, double (&v)[RPL]) {
 #pragma unroll
@@ -261,7 +282,7 @@ __device__ __forceinline__ void pair_resum(const PhiArgs &a, int nm1, int K, int
     for (int p = q - 1; more; --p) {
         more = p > qa && !((__ldg(a.rstart + (p >> 5)) >> (p & 31)) & 1u);
         double pv[RPL];
-        double d = pair_row64<RPL, G, PI>(a, nm1, K, p, row, lane, pv);
+        double d = pair_row64<NM1, RPL, G, PI>(a, nm1, K, p, row, lane, pv);
 #pragma unroll
         for (int o = G / 2; o > 0; o >>= 1) d += __shfl_xor_sync(gmask, d, o);
         d = phi_divide(__ldg(reinterpret_cast<const double *>(a.val) + p), d, a.eps);
@@ -400,7 +421,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
                 if (((esc >> r) & 1u) && !(v[r] >= bound)) low |= 1u << r;
         }
         if (__builtin_expect(__any_sync(gmask, low != 0u), 0)) {
-            pair_resum<RPL, G, PI>(a, nm1, K, qa, q, cur, lane, gmask, low, v);
+            pair_resum<NM1, RPL, G, PI>(a, nm1, K, qa, q, cur, lane, gmask, low, v);
         }
 #pragma unroll
         for (int r = 0; r < RPL; ++r) v[r] = scale_pow2(v[r], -SC);
@@ -475,7 +496,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
             uint32_t bad = 0;
 #pragma unroll
             for (int v = 0; v < VP; ++v) {
-                PairProduct y0, y1;
+                PairProduct<true> y0, y1;
 #pragma unroll
                 for (int k = 0; k < MAXK; ++k) {
                     if (k < nm1) {
@@ -498,6 +519,19 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
                 bad |= (y1.pair_ok() || y1.zero() ? 0u : 1u) << (2 * v + 1);
             }
             if (__builtin_expect(bad != 0u, 0)) {
+                // an element below the window for certain needs no value here: an escape
+                // of 0 leaves it out like any small one, and pair_resum forms it where it
+                // matters (with the FP64 product of each, a quarter of all elements along
+                // a solve, launches of the 3-way tensor grew from 0.85 to 4.8 ms in 24 outer
+                // iterations; now to 3.2)
+#pragma unroll
+                for (int r = 0; r < RPL; ++r) {
+                    float &h = r % 2 ? ph[u][r / 2].y : ph[u][r / 2].x;
+                    if (((bad >> r) & 1u) && fabsf(h) < 0.5f * kPairLowF) {
+                        h = __uint_as_float(0x80000000u);
+                        bad &= ~(1u << r);
+                    }
+                }
 #pragma unroll
                 for (int r = 0; r < RPL; ++r)
                     if ((bad >> r) & 1u) {
@@ -616,7 +650,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
 #pragma unroll 1
             for (int u = 0; u < U; ++u)
                 if (__any_sync(full, (redo >> u) & 1u))
-                    ll += pair_redo<RPL, G, OP, PI>(a, acc, nm1, K, min(q + u, p1 - 1), cur, lane, (redo >> u) & 1u);
+                    ll += pair_redo<NM1, RPL, G, OP, PI>(a, acc, nm1, K, min(q + u, p1 - 1), cur, lane, (redo >> u) & 1u);
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if ((redo >> u) & 1u) {

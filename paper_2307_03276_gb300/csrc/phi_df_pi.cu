@@ -36,14 +36,14 @@ __global__ void __launch_bounds__(256) pair_factor_kernel(const double2 *__restr
     if (blockIdx.x == 0 && threadIdx.x == 0) *kexp = k;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nv; e += (int64_t)gridDim.x * blockDim.x) {
         const double2 x = A[e];
-        const float2 p = pair_encode(x.x, c - k, c), q = pair_encode(x.y, c - k, c);
+        const float2 p = pair_factor(x.x, c - k, c), q = pair_factor(x.y, c - k, c);
         P[e] = make_float4(p.x, q.x, p.y, q.y);
     }
 }
 
 // Khatri-Rao rows of one mode as pairs, like pi_build_range: one thread per
 // 16-byte vector (two elements).  The products are formed as the fused kernel
-// forms them (load_rows in df_walk), so the two give the same bits.
+// forms them (form_rows in df_walk), so the two give the same bits.
 template <int NM1>
 __global__ void __launch_bounds__(256) pi_pair_kernel(const PhiArgs a, float4 *__restrict__ pi) {
     constexpr int MAXK = NM1 > 0 ? NM1 : kMaxNm1;
@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(256) pi_pair_kernel(const PhiArgs a, float4 *_
         const int64_t p = e >> lg;
         const int v = (int)(e & (vpr - 1));
         int32_t ii[MAXK];
-        PairProduct q0, q1;
+        PairProduct<false> q0, q1;
 #pragma unroll
         for (int k = 0; k < MAXK; ++k) {
             if (k < nm1) {

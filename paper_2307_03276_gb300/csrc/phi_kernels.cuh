@@ -36,6 +36,11 @@
 // whoever writes a final Phi row also reduces its violation, and one atomicMax
 // per block publishes it (non-negative doubles order like their bit patterns).
 //
+// Which launches run this kernel: FP64 Phi below a wave of tiles, FP64 MTTKRP,
+// the fused log-likelihood and 3-way FP32 MTTKRP.  Large FP64 Phi launches work on
+// float pairs (df_walk.cuh) and the other FP32 launches in direct.cuh; both share
+// the three levels above (segmented_tail) and the violation.
+//
 // FP32 form: gathers, Khatri-Rao products, dot and scale in FP32; a run of
 // same-row nonzeros is summed in plain FP32 over two interleaved
 // accumulators, the sums of partial rows across groups and tiles are
