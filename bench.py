@@ -20,7 +20,7 @@ design.
 
 Reported beside it: the FP32 form of the same step, the FP64 step with the
 Khatri-Rao rows formed in place, the 3-way tensor's FP64 and FP32 steps, the
-roofline of the dominant kernel (the Phi tile kernel), an end-to-end number
+roofline of the dominant kernel (the Phi kernel), an end-to-end number
 through the C ABI from pinned host buffers, MTTKRP kernel throughput, the
 batched solver, the time to KKT tolerance 1e-4 (a small tensor solved to the
 tolerance, the headline tensor to a violation level FP64 and FP32 both
@@ -598,7 +598,7 @@ def on_pairs(T, info) -> bool:
 
 
 def roofline_for(T, inner_per_mode, stats, precision, peaks, cp, pi_modes=None, info=None, pairs=False):
-    """Roofline of the Phi tile kernel from its measured average duration.
+    """Roofline of the Phi kernel from its measured average duration.
     pi_modes: per mode, whether Phi streamed materialised Khatri-Rao rows.
     pairs: FP64 on float-pair rows, no FP64 arithmetic per element: HBM is the bound."""
     N, nnz, R = T.nmodes, T.nnz, T.rank
