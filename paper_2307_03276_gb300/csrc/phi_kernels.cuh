@@ -1089,13 +1089,22 @@ __device__ __forceinline__ void pi_build_range(const PhiArgs &a, T *__restrict__
     for (int64_t e = e0; e < e1; e += step) {
         const int64_t p = e >> lg;
         const int c = (int)(e & (vpr - 1)) * VN;
-        V x = __ldg(reinterpret_cast<const V *>(reinterpret_cast<const T *>(a.A[0]) +
-                                                (int64_t)__ldg(a.idx[0] + p) * a.Rp + c));
+        // coordinates first (FP32, 5 modes, 9e6 nonzeros, R = 32: 0.367 against 0.495 ms a
+        // mode; 3 modes 0.031, 0.033), but with three gathered factors each beside its
+        // entries (4 modes, 2e7, R = 16: 0.348 against 0.381 ms)
+        int32_t ii[MAXK];
+        if constexpr (NM1 != 3) {
+#pragma unroll
+            for (int k = 0; k < MAXK; ++k)
+                if (k < nm1) ii[k] = __ldg(a.idx[k] + p);
+        }
+        auto at = [&](int k) -> int32_t { return NM1 != 3 ? ii[k] : __ldg(a.idx[k] + p); };
+        V x = __ldg(reinterpret_cast<const V *>(reinterpret_cast<const T *>(a.A[0]) + (int64_t)at(0) * a.Rp + c));
 #pragma unroll
         for (int k = 1; k < MAXK; ++k) {
             if (k < nm1) {
                 const V y = __ldg(reinterpret_cast<const V *>(reinterpret_cast<const T *>(a.A[k]) +
-                                                              (int64_t)__ldg(a.idx[k] + p) * a.Rp + c));
+                                                              (int64_t)at(k) * a.Rp + c));
                 if constexpr (VN == 4) {
                     x.x *= y.x;
                     x.y *= y.y;
