@@ -17,6 +17,10 @@
  *  - Pointers may be host (pageable or pinned) or device pointers; the
  *    library tells them apart through unified addressing.  Inputs are
  *    copied: the caller keeps ownership of every buffer it passes.
+ *  - Device (and managed) inputs are read after all work queued on the legacy
+ *    default stream before the call.  Work on any other stream that writes an
+ *    input, or still uses an output buffer, must have finished before the call
+ *    (an output buffer: on the default stream too).
  *  - Outputs are complete when the call returns (the call synchronises its
  *    stream before returning).
  *  - Errors are returned as cpapr_status; no exception crosses the ABI.  A

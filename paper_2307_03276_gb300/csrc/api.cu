@@ -456,6 +456,7 @@ void cpapr_destroy(cpapr_ctx *ctx) {
         cudaEventDestroy(p.second.second);
     }
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
+    if (ctx->caller_done) cudaEventDestroy(ctx->caller_done);
     if (ctx->own_stream && ctx->stream) cudaStreamDestroy(ctx->stream);
     host_slot_release(ctx->host);
     delete ctx;
@@ -515,6 +516,8 @@ cpapr_status cpapr_create(int32_t nmodes, const int64_t *dims, int64_t nnz, cons
         if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "cudaStreamCreate"));
         ctx->own_stream = true;
     }
+    e = cudaEventCreateWithFlags(&ctx->caller_done, cudaEventDisableTiming);
+    if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "cudaEventCreate"));
     const int Rp = ctx->Rp;
     void *p = nullptr;
     cpapr_status st;

@@ -427,6 +427,9 @@ cpapr_status build_layouts(cpapr_ctx *ctx, const int64_t *const *idx_in, const d
         const int64_t *src[kMaxModes] = {};
         for (int m = 0; m < N; ++m) src[m] = static_cast<const int64_t *>(device_view(idx_in[m]));
         const double *vsrc = static_cast<const double *>(device_view(vals_in));
+        const void *in[kMaxModes + 1] = {vals_in};
+        for (int m = 0; m < N; ++m) in[m + 1] = idx_in[m];
+        BL_TRY(wait_for_caller(ctx, in, N + 1));
         for (int m = 0; m < N; ++m) {
             if (!src[m]) BL_CUDA(lib_malloc((void **)&stage[m], nb * 8, s));
             BL_CUDA(lib_malloc((void **)&idx32[m], nb * 4, s));

@@ -96,6 +96,7 @@ struct cpapr_ctx {
     cpapr_options opt{};
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    cudaEvent_t caller_done = nullptr;  // wait_for_caller
     int device = 0;
     size_t esize = 8;  // bytes per element of the working precision
     cpapr::ModeLayout mode[CPAPR_MAX_MODES];
@@ -268,6 +269,10 @@ cpapr_status download_matrix(cpapr_ctx *ctx, const void *src, int64_t rows, doub
 cpapr_status launch_set_model(cpapr_ctx *ctx, const double *lambda, const double *const *factors);
 // memory of the context's device (or managed) that a kernel may read or write as doubles in place
 bool device_doubles(const cpapr_ctx *ctx, const void *p);
+// before the context's stream reads the caller's p: if it is device or managed memory,
+// the stream waits for what the caller has queued on the legacy default stream
+cpapr_status wait_for_caller(cpapr_ctx *ctx, const void *p);
+cpapr_status wait_for_caller(cpapr_ctx *ctx, const void *const *p, int n);
 cpapr_status launch_kkt_rows(cpapr_ctx *ctx, int n, const void *B, const void *Phi, InnerState *inner);
 
 // ---- small utilities (index.cu) ---------------------------------------------

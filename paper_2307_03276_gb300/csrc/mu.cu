@@ -461,7 +461,31 @@ bool device_doubles(const cpapr_ctx *ctx, const void *p) {
            ((uintptr_t)p & 7) == 0;
 }
 
+// The context's own stream does not synchronise with the legacy default stream
+// (cudaStreamNonBlocking), where a caller's framework may just have queued the
+// kernels that write p: an event there orders the reads after them without a host
+// wait.  Work on the caller's other streams is the caller's to order.
+cpapr_status wait_for_caller(cpapr_ctx *ctx, const void *const *p, int n) {
+    for (int k = 0; k < n; ++k) {
+        cudaPointerAttributes t;
+        if (cudaPointerGetAttributes(&t, p[k]) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (t.type != cudaMemoryTypeDevice && t.type != cudaMemoryTypeManaged) continue;
+        CPAPR_CUDA(ctx, cudaEventRecord(ctx->caller_done, cudaStreamLegacy));
+        CPAPR_CUDA(ctx, cudaStreamWaitEvent(ctx->stream, ctx->caller_done, 0));
+        return CPAPR_OK;
+    }
+    return CPAPR_OK;
+}
+
+cpapr_status wait_for_caller(cpapr_ctx *ctx, const void *p) { return wait_for_caller(ctx, &p, 1); }
+
 cpapr_status launch_set_model(cpapr_ctx *ctx, const double *lambda, const double *const *factors) {
+    const void *in[kMaxModes + 1] = {lambda};
+    for (int m = 0; m < ctx->N; ++m) in[m + 1] = factors[m];
+    CPAPR_TRY(wait_for_caller(ctx, in, ctx->N + 1));
     ModelArgs a{};
     a.R = ctx->R;
     a.Rp = ctx->Rp;
@@ -511,6 +535,7 @@ cpapr_status launch_set_model(cpapr_ctx *ctx, const double *lambda, const double
 static cpapr_status upload_matrix2(cpapr_ctx *ctx, const double *src, int64_t rows, void *dst, double *dst64) {
     const int R = ctx->R, Rp = ctx->Rp;
     const int64_t n = rows * Rp;
+    CPAPR_TRY(wait_for_caller(ctx, src));
     CPAPR_CUDA(ctx, cudaMemsetAsync(ctx->stage, 0, (size_t)n * 8, ctx->stream));
     if (rows > 0)
         CPAPR_CUDA(ctx, cudaMemcpy2DAsync(ctx->stage, (size_t)Rp * 8, src, (size_t)R * 8, (size_t)R * 8, (size_t)rows,
