@@ -112,11 +112,12 @@ template <typename T> struct KSum {
 template <> struct KSum<float> {
     float s, c;
     __device__ __forceinline__ void zero() { s = 0.f; c = 0.f; }
-    // Kahan (1965): carry the rounding error of every addition in c
+    // Kahan (1965): carry the rounding error of every addition in c (none for a sum
+    // that overflows: it stays infinite, where its correction would make it NaN)
     __device__ __forceinline__ void add(float x) {
         float y = x - c;
         float t = s + y;
-        c = (t - s) - y;
+        c = fabsf(t) < __int_as_float(0x7f800000) ? (t - s) - y : 0.f;
         s = t;
     }
     __device__ __forceinline__ void fma_add(float v, float p) { add(v * p); }
