@@ -25,7 +25,7 @@
 #include "internal.cuh"
 
 namespace cpapr {
-cpapr_status launch_phi_given_carry(cpapr_ctx *ctx, int n, const void *B, void *out, void *carry);
+cpapr_status launch_phi_given_carry(cpapr_ctx *ctx, int n, const void *B, void *out, void *carry, int sh);
 }
 
 using namespace cpapr;
@@ -89,8 +89,15 @@ extern "C" cpapr_status cpapr_phi_noalloc(cpapr_ctx *ctx, int32_t mode, const do
     if (!out || !is_device_pointer(out)) return fail(ctx, CPAPR_E_ARG, "out must be a device pointer");
     if (B && !is_device_pointer(B)) return fail(ctx, CPAPR_E_ARG, "B must be NULL or a device pointer");
     const ModeLayout &L = ctx->mode[mode];
-    const int64_t tiles = ceil_div(ctx->nnz, (int64_t)L.tile_nnz << phi_shift(ctx, mode));
-    const int64_t need = 2 * tiles * ctx->Rp * (int64_t)ctx->esize;
+    // cpapr_phi's tiles, or those of the mode's other launches where only these fit the
+    // scratch (padded rank 128 over float pairs: 512 nonzeros, and 1024)
+    int sh = phi_shift(ctx, mode);
+    auto scratch_for = [&](int k) {
+        return 2 * ceil_div(ctx->nnz, (int64_t)L.tile_nnz << k) * ctx->Rp * (int64_t)ctx->esize;
+    };
+    if (scratch_for(sh) > (int64_t)CPAPR_NOALLOC_SCRATCH_BYTES) sh = std::max(sh, L.sh);
+    const int64_t need = scratch_for(sh);
+    const int64_t tiles = ceil_div(ctx->nnz, (int64_t)L.tile_nnz << sh);
     if (need > (int64_t)CPAPR_NOALLOC_SCRATCH_BYTES)
         return fail(ctx, CPAPR_E_RANGE,
                     "cpapr_phi_noalloc: this mode needs " + std::to_string(need) + " bytes of scratch (2 x " +
@@ -114,7 +121,7 @@ extern "C" cpapr_status cpapr_phi_noalloc(cpapr_ctx *ctx, int32_t mode, const do
         // is cleared (the materialised rows, if the mode uses them, live in
         // the context's buffer and are rebuilt for this call)
         CPAPR_TRY(prepare_phi(ctx, mode));
-        CPAPR_TRY(launch_phi_given_carry(ctx, mode, ctx->B, ctx->outbuf, scratch));
+        CPAPR_TRY(launch_phi_given_carry(ctx, mode, ctx->B, ctx->outbuf, scratch, sh));
         CPAPR_TRY(download_matrix(ctx, ctx->outbuf, ctx->dims[mode], out));
     }
     // Did a tile's bounded staging wait give up?  Such a tile never wrote its

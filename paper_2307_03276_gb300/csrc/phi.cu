@@ -307,16 +307,16 @@ cpapr_status launch_phi(cpapr_ctx *ctx, int n, PhiOp op, const void *B, void *ou
     return CPAPR_OK;
 }
 
-// Phi^(n) with the segmented reduction and a caller-supplied carry buffer
-// (2 x ntiles x Rp elements of the working type).  Launches kernels only:
-// no allocation, no event, no memset.
-cpapr_status launch_phi_given_carry(cpapr_ctx *ctx, int n, const void *B, void *out, void *carry) {
+// Phi^(n) with the segmented reduction over tiles of 2^sh table tiles and a
+// caller-supplied carry buffer (2 x tiles x Rp elements of the working type).
+// Launches kernels only: no allocation, no event, no memset.
+cpapr_status launch_phi_given_carry(cpapr_ctx *ctx, int n, const void *B, void *out, void *carry, int sh) {
     ModeLayout &L = ctx->mode[n];
     PhiArgs a = make_args(ctx, n, B, out, nullptr);
     a.atomic = 0;
     a.carry = carry;
     if (L.pi) a.pi = ctx->pibuf;
-    set_tiles(a, L, phi_shift(ctx, n));
+    set_tiles(a, L, sh);
     if (ctx->nnz == 0) return fail(ctx, CPAPR_E_ARG, "empty tensor");
     CPAPR_TRY(launch_zero_empty(ctx, n, out));
     cudaError_t e = dispatch(ctx, a, ctx->Rp / L.lanes, L.lanes, OP_PHI);
