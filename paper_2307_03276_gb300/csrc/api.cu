@@ -327,7 +327,7 @@ cpapr_status configure_mode(cpapr_ctx *ctx, int n, int lanes, int tile, int redu
         cudaGraphExecDestroy(ctx->graph_exec[n]);
         ctx->graph_exec[n] = nullptr;
     }
-    return ensure_pair_storage(ctx);
+    return CPAPR_OK;
 }
 
 // Materialised Khatri-Rao rows: one buffer of nnz_pad x Rp elements shared by
@@ -597,10 +597,11 @@ cpapr_status cpapr_create(int32_t nmodes, const int64_t *dims, int64_t nnz, cons
             ctx->mode[n].sh = h.sh;
             ctx->mode[n].sh_df = h.sh_df;
             ctx->mode[n].batch_sh = h.batch_sh;
-            CR_TRY(ensure_pair_storage(ctx));
         }
         CR_TRY(configure_pi(ctx, n, pi));
     }
+    // after everything the context cannot do without
+    CR_TRY(ensure_pair_storage(ctx));
     if (o.autotune || o.tune_cache) CR_TRY(autotune(ctx));
     ctx->opt.tune_cache = nullptr;  // the caller's string is not kept
     e = cudaStreamSynchronize(ctx->stream);

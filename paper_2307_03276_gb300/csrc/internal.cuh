@@ -223,7 +223,7 @@ enum PhiOp { OP_PHI = 0, OP_MTTKRP = 1, OP_LL = 2 };
 // B: I_n x Rp of the working type (ignored for MTTKRP).  inner: state whose
 // done flag / kkt slot the kernels use (may be null for a one-off Phi).
 cpapr_status launch_phi(cpapr_ctx *ctx, int n, PhiOp op, const void *B, void *out, InnerState *inner);
-// does Phi of mode n run on float pairs (df_pair.cuh)?  Allocates their storage if so.
+// does Phi of mode n run on float pairs (df_pair.cuh)?
 bool uses_pairs(const cpapr_ctx *ctx, int n);
 // log2 of the table tiles per tile of mode n's Phi launch
 inline int phi_shift(const cpapr_ctx *ctx, int n) {

@@ -105,7 +105,7 @@ uint32_t injected_stage_shortfall() {
 // scales cover, and faster where the launch has at least a wave of tiles (4 per
 // SM); a launch of a few tiles is bound by one tile's latency, which the longer
 // FP32 instruction chains raise.
-bool uses_pairs(const cpapr_ctx *ctx, int n) {
+static bool pairs_apply(const cpapr_ctx *ctx, int n) {
     const ModeLayout &L = ctx->mode[n];
     const int dot = ctx->opt.fp64_dot;
     if (L.tile_nnz == 0) return false;  // not configured yet
@@ -115,14 +115,23 @@ bool uses_pairs(const cpapr_ctx *ctx, int n) {
             (dot == CPAPR_DOT_AUTO && ceil_div(ctx->nnz, (int64_t)L.tile_nnz << L.sh) >= kDfMinTiles));
 }
 
+bool uses_pairs(const cpapr_ctx *ctx, int n) { return ctx->P[0] && pairs_apply(ctx, n); }
+
+// The factors as pairs, where some mode's Phi would read them.  A context without
+// the room for them (8 bytes per padded factor entry) keeps the kernels that need none.
 cpapr_status ensure_pair_storage(cpapr_ctx *ctx) {
     bool any = false;
-    for (int n = 0; n < ctx->N; ++n) any = any || uses_pairs(ctx, n);
+    for (int n = 0; n < ctx->N; ++n) any = any || pairs_apply(ctx, n);
     if (!any || ctx->P[0]) return CPAPR_OK;
     size_t ofs[CPAPR_MAX_MODES + 1] = {};
     for (int m = 0; m < ctx->N; ++m) ofs[m + 1] = ofs[m] + (((size_t)ctx->dims[m] * ctx->Rp * 8 + 255) & ~(size_t)255);
     void *p = nullptr;
-    CPAPR_TRY(dev_alloc(ctx, &p, ofs[ctx->N] + 256));
+    const cpapr_status st = dev_alloc(ctx, &p, ofs[ctx->N] + 256);
+    if (st == CPAPR_E_NOMEM) {
+        ctx->err.clear();
+        return CPAPR_OK;
+    }
+    CPAPR_TRY(st);
     char *base = (char *)p;
     ctx->pair_top = (unsigned long long *)(base + ofs[ctx->N]);
     ctx->kexp = (int32_t *)(base + ofs[ctx->N] + 128);
