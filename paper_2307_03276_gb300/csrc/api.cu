@@ -709,6 +709,10 @@ cpapr_status cpapr_set_state(cpapr_ctx *ctx, const double *lambda, const double 
         }
     }
     ctx->k_total = outer_done;
+    // after an outer iteration every factor is normalised: the pairs' exponents are
+    // those of the solve that goes on, not measured again (as for a model just set)
+    if (outer_done > 0)
+        for (int m = 0; m < ctx->N; ++m) ctx->pair_state[m] = kPairNormalised;
     return CPAPR_OK;
 }
 
