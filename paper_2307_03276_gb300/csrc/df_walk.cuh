@@ -16,8 +16,8 @@
 // open: loads of the next step, and the block's slowest warp at a tile's end.
 //
 // Scaled quantities (all powers of two): pi' = pi 2^K (the pairs), b' = b 2^(S - K),
-// eps' = eps 2^S, s' = s 2^S with S = kDfS; v' = v 2^V with V = kDfV; sums of
-// v' pi' carry 2^(K + V).  The float range then covers
+// eps' = eps 2^S, s' = s 2^S with S = kDfS; v' = v 2^V with V = kDfV; FP32 sums
+// of v' pi' carry 2^(K + V), the FP64 accumulators nothing.  The float range then covers
 //   pi' in [2^-80, 2^67], v' in [2^-20, 2^50] or 0, s' in [0, 2^100);
 // a nonzero outside (a huge model value, a count outside {0} and [2^-20, 2^31), a
 // quotient outside the window) is redone in FP64 by its group.  Escaped elements
@@ -262,8 +262,8 @@ __device__ __forceinline__ double pair_redo(const PhiArgs &a, double2 *acc, int 
 #pragma unroll
     for (int k = 0; k < RPL / 2; ++k) {
         double2 t = acc[k * G + lane];
-        t.x += scale_pow2(v * pv[2 * k], K + kDfV);
-        t.y += scale_pow2(v * pv[2 * k + 1], K + kDfV);
+        t.x = fma(v, pv[2 * k], t.x);
+        t.y = fma(v, pv[2 * k + 1], t.y);
         acc[k * G + lane] = t;
     }
     return 0.0;
@@ -288,7 +288,7 @@ __device__ __forceinline__ void pair_resum(const PhiArgs &a, int nm1, int K, int
         d = phi_divide(__ldg(reinterpret_cast<const double *>(a.val) + p), d, a.eps);
 #pragma unroll
         for (int r = 0; r < RPL; ++r)
-            if ((low >> r) & 1u) v[r] += scale_pow2(d * pv[r], K + kDfV);
+            if ((low >> r) & 1u) v[r] = fma(d, pv[r], v[r]);
     }
 }
 
@@ -343,7 +343,9 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
     int K = nm1 * pair_scale(nm1);
     for (int m = 0; m <= nm1; ++m)
         if (m != a.mode) K -= __ldg(a.kexp + m);
-    const int SC = K + kDfV;  // the sums carry 2^SC
+    // the FP32 sums carry 2^(K + kDfV), the FP64 accumulator nothing, so that it has the
+    // FP64 range (|K| <= 760); unit takes the one to the other, exactly
+    const double unit = __hiloint2double((1023 - K - kDfV) << 20, 0);
     float eh, el;
     df_cut(a.eps, kDfS, eh, el);
     const float bmax = eh * 0x1p34f;
@@ -406,8 +408,8 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
 #pragma unroll
         for (int k = 0; k < VP; ++k) {
             const double2 t = acc[k * G + lane];
-            v[2 * k] = t.x + (df_widen(S[k].x) + df_widen(C[k].x));
-            v[2 * k + 1] = t.y + (df_widen(S[k].y) + df_widen(C[k].y));
+            v[2 * k] = fma(df_widen(S[k].x) + df_widen(C[k].x), unit, t.x);
+            v[2 * k + 1] = fma(df_widen(S[k].y) + df_widen(C[k].y), unit, t.y);
             acc[k * G + lane] = make_double2(0.0, 0.0);
             S[k] = C[k] = make_float2(0.f, 0.f);
         }
@@ -415,7 +417,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
         // beside a sum of 2^-25 of them or more; a column with less is summed again
         uint32_t low = 0;
         if (__builtin_expect(esc != 0u, 0)) {
-            const double bound = df_widen(__uint_as_float(esc & ~0xffu)) * 0x1p-25;
+            const double bound = df_widen(__uint_as_float(esc & ~0xffu)) * 0x1p-25 * unit;
 #pragma unroll
             for (int r = 0; r < RPL; ++r)
                 if (((esc >> r) & 1u) && !(v[r] >= bound)) low |= 1u << r;
@@ -423,8 +425,6 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
         if (__builtin_expect(__any_sync(gmask, low != 0u), 0)) {
             pair_resum<NM1, RPL, G, PI>(a, nm1, K, qa, q, cur, lane, gmask, low, v);
         }
-#pragma unroll
-        for (int r = 0; r < RPL; ++r) v[r] = scale_pow2(v[r], -SC);
         esc = 0;
         if (!before && !after) {
             double *o = out + (int64_t)cur * Rp;
@@ -683,8 +683,8 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
 #pragma unroll
                 for (int k = 0; k < VP; ++k) {
                     double2 t = acc[k * G + lane];
-                    t.x += df_widen(S[k].x) + df_widen(C[k].x);
-                    t.y += df_widen(S[k].y) + df_widen(C[k].y);
+                    t.x = fma(df_widen(S[k].x) + df_widen(C[k].x), unit, t.x);
+                    t.y = fma(df_widen(S[k].y) + df_widen(C[k].y), unit, t.y);
                     acc[k * G + lane] = t;
                     S[k] = C[k] = make_float2(0.f, 0.f);
                 }
