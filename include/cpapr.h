@@ -99,7 +99,7 @@ enum { CPAPR_DOT_AUTO = 0, CPAPR_DOT_FP64 = 1, CPAPR_DOT_FP32_PIPE = 2 };
  *             scaled addition; Phi's error stays below 1e-12 relative per entry
  *             (measured near 1e-14).  It applies where rank_lanes leaves 8 or
  *             fewer ranks per lane and 2^-43 <= eps <= 2^20; a nonzero outside
- *             its ranges (a value outside {0} and [2^-20, 2^31), ...) is
+ *             its ranges (a value outside {0} and [2^-20, 2^30), ...) is
  *             evaluated in FP64.  CPAPR_DOT_AUTO (default): the FP32 pipe where
  *             the tensor has at least 608 tiles (4 per SM; of 2048 nonzeros, 1024
  *             from rank 17 on, or of tile_nnz), FP64 below that, where one tile's

@@ -19,7 +19,7 @@
 // eps' = eps 2^S, s' = s 2^S with S = kDfS; v' = v 2^V with V = kDfV; FP32 sums
 // of v' pi' carry 2^(K + V), the FP64 accumulators nothing.  The float range then covers
 //   pi' in [2^-80, 2^67], v' in [2^-20, 2^50] or 0, s' in [0, 2^100);
-// a nonzero outside (a huge model value, a count outside {0} and [2^-20, 2^31), a
+// a nonzero outside (a huge model value, a count outside {0} and [2^-20, 2^30), a
 // quotient outside the window) is redone in FP64 by its group.  Escaped elements
 // add 0 to the dot: they are below 2^-80 while max(s', eps') >= eps', so the
 // dropped terms stay below 2^-47 of it where b' < eps' 2^34; else the nonzero is
@@ -44,6 +44,7 @@ namespace cpapr {
 
 constexpr int kDfS = 60;
 constexpr int kDfV = 10;
+static_assert(30 + kDfS + kDfV <= 100, "df_bad_x: counts below 2^30 stay below df_cut's 2^100");
 constexpr int kDfThreads = 128;
 // Resident blocks per SM the registers are held to (96 each).  4 / 5 / 6 blocks:
 // 1.43 / 1.31 / 1.36 ms a launch (4-way, 5e7 nonzeros, R = 16), 0.64 / 0.58 / 0.59 ms
@@ -143,11 +144,11 @@ __device__ __forceinline__ float2 df_divide(float xh, float xl, float2 s, float 
     return make_float2(h, q1 - (h - q0));
 }
 
-// true unless x = 0 or 2^-20 <= x < 2^31 (x >= 0)
+// true unless x = 0 or 2^-20 <= x < 2^30 (x >= 0): x 2^(kDfS + kDfV) is within df_cut's range
 __device__ __forceinline__ bool df_bad_x(double x) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
     const unsigned e = (unsigned)(bits >> 52);
-    return bits != 0ull && (e < 1023u - 20u || e >= 1023u + 31u);
+    return bits != 0ull && (e < 1023u - 20u || e >= 1023u + 30u);
 }
 
 // the reduce-scatter of group_reduce_scatter for pairs, over the whole warp

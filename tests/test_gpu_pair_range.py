@@ -55,3 +55,18 @@ def test_sums_far_below_the_largest_products(pi_mode):
         want = oracle.phi(dims, idx, vals, fs, fs[0], 0)
         assert 0 < want[::2][want[::2] > 0].min() < 1e-200
         check(t.phi(0), want)
+
+
+@pytest.mark.parametrize("pi_mode", PI)
+def test_counts_at_the_edges_of_the_quotients_range(pi_mode):
+    """Counts from 2^-20 up to 2^30 take the FP32 quotient, all others FP64."""
+    dims, rank = (50, 40, 30), 8
+    rng, idx, vals = tensor(dims, 3000, 3)
+    fs = [0.5 + 0.5 * rng.random((d, rank)) for d in dims]
+    edge = np.array([2.0 ** -20, np.nextafter(2.0 ** -20, 0), np.nextafter(2.0 ** 30, 0), 2.0 ** 30, 2.0 ** 30 - 1, 2.0 ** 31])
+    vals[:] = edge[rng.integers(0, edge.size, vals.size)]
+    vals[::11] = 0.0
+    with cpapr.Tensor(dims, idx, vals, rank, fp64_dot=cpapr.CPAPR_DOT_FP32_PIPE, pi_mode=pi_mode) as t:
+        t.set_model(np.ones(rank), fs)
+        for n in range(3):
+            check(t.phi(n), oracle.phi(dims, idx, vals, fs, fs[n], n))
