@@ -18,10 +18,10 @@
 // Scaled quantities (all powers of two): pi' = pi 2^K (the pairs), b' = b 2^(S - K),
 // eps' = eps 2^S, s' = s 2^S with S = kDfS; v' = v 2^V with V = kDfV; FP32 sums
 // of v' pi' carry 2^(K + V), the FP64 accumulators nothing.  The float range then covers
-//   pi' in [2^-80, 2^67], v' in [2^-20, 2^50] or 0, s' in [0, 2^100);
+//   pi' in [2^-80, 2^60], v' in [2^-20, 2^50] or 0, s' in [0, 2^100);
 // a nonzero outside (a huge model value, a count outside {0} and [2^-20, 2^30), a
 // quotient outside the window) is redone in FP64 by its group.  Escaped elements
-// add 0 to the dot: they are below 2^-80 while max(s', eps') >= eps', so the
+// below the window add 0 to the dot: they are below 2^-80 while max(s', eps') >= eps', so the
 // dropped terms stay below 2^-47 of it where b' < eps' 2^34; else the nonzero is
 // redone in FP64.  They are left out of the sums as well, with a bound on what
 // that leaves out; a column whose sum is not large beside it is summed again in
@@ -179,37 +179,39 @@ __device__ __forceinline__ float2 group_reduce_scatter_df(float2 (&s)[U], int la
 // they cost the loop its registers, 1.53 against 1.39 ms a launch on the 4-way
 // tensor.)
 
-// an element of a row formed in place as the pairs hold it, from the FP64 factors
-__device__ __forceinline__ float2 pair_exact(const PhiArgs &a, int nm1, int K, int p, int c) {
-    double d = 0.0;
-#pragma unroll 1
-    for (int k = 0; k < nm1; ++k) {
-        const int32_t i = __ldg(a.idx[k] + p);
-        const double f = __ldg(reinterpret_cast<const double *>(a.A[k]) + (int64_t)i * a.Rp + c);
-        d = k == 0 ? f : d * f;
-    }
-    return pair_encode(d, K, kPairMax);
-}
-
-// this lane's columns of nonzero p's row in FP64, and its part of <B[row], pi>; a row
-// formed in place loads all its coordinates, then all its factor entries, at once
+// this lane's columns of nonzero p's row in FP64, and its part of <B[row], pi>: the
+// pairs' values, and FP64 products where there is none
 template <int NM1, int RPL, int G, bool PI>
 __device__ __forceinline__ double pair_row64(const PhiArgs &a, int nm1, int K, int p, int row, int lane,
                                              double (&pv)[RPL]) {
     const double *B = reinterpret_cast<const double *>(a.B) + (int64_t)row * (RPL * G);
-    constexpr int Rp = RPL * G, MAXK = NM1 > 0 ? NM1 : kMaxNm1;
-    double d = 0.0;
-    if constexpr (PI) {
-#pragma unroll
-        for (int r = 0; r < RPL; ++r)
-            pv[r] = pair_value(pair_at(reinterpret_cast<const float *>(a.pi), (int64_t)p * Rp, ((r >> 1) * G + lane) * 2 + (r & 1)), K);
-    } else {
-        int64_t at[MAXK];
+    constexpr int Rp = RPL * G, MAXK = PI ? 1 : NM1 > 0 ? NM1 : kMaxNm1;
+    int64_t at[MAXK];
+    if constexpr (!PI) {
 #pragma unroll
         for (int k = 0; k < MAXK; ++k) at[k] = k < nm1 ? (int64_t)__ldg(a.idx[k] + p) * Rp : 0;
+    }
 #pragma unroll
-        for (int v = 0; v < RPL / 2; ++v) {
-            PairProduct<true> y0, y1;
+    for (int v = 0; v < RPL / 2; ++v) {
+        float2 e0, e1;
+        double2 f = make_double2(0.0, 0.0);
+        if constexpr (PI) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int c = (v * G + lane) * 2 + h;
+                const float2 e = pair_at(reinterpret_cast<const float *>(a.pi), (int64_t)p * Rp, c);
+                double d = pair_value(e, K);
+                if (is_escape(e)) {
+                    d = 1.0;
+#pragma unroll 1
+                    for (int k = 0; k < nm1; ++k)
+                        d *= __ldg(reinterpret_cast<const double *>(a.A[k]) + (int64_t)__ldg(a.idx[k] + p) * Rp + c);
+                }
+                pv[2 * v + h] = d;
+            }
+            continue;
+        } else {
+            PairProduct y0, y1;
 #pragma unroll
             for (int k = 0; k < MAXK; ++k)
                 if (k < nm1) {
@@ -222,11 +224,9 @@ __device__ __forceinline__ double pair_row64(const PhiArgs &a, int nm1, int K, i
                         y1.mul(make_float2(y.y, y.w));
                     }
                 }
-            if (y0.zero()) y0.p = make_float2(0.f, 0.f);
-            if (y1.zero()) y1.p = make_float2(0.f, 0.f);
-            const bool ok0 = y0.pair_ok() || y0.zero(), ok1 = y1.pair_ok() || y1.zero();
-            if (!(ok0 && ok1)) {
-                double2 f = make_double2(0.0, 0.0);
+            e0 = y0.value();
+            e1 = y1.value();
+            if (is_escape(e0) || is_escape(e1)) {
 #pragma unroll
                 for (int k = 0; k < MAXK; ++k)
                     if (k < nm1) {
@@ -234,13 +234,12 @@ __device__ __forceinline__ double pair_row64(const PhiArgs &a, int nm1, int K, i
                                                     reinterpret_cast<const double *>(a.A[k]) + at[k]) + v * G + lane);
                         f = k == 0 ? g : make_double2(f.x * g.x, f.y * g.y);
                     }
-                if (!ok0) y0.p = pair_encode(f.x, K, kPairMax);
-                if (!ok1) y1.p = pair_encode(f.y, K, kPairMax);
             }
-            pv[2 * v] = pair_value(y0.p, K);
-            pv[2 * v + 1] = pair_value(y1.p, K);
         }
+        pv[2 * v] = is_escape(e0) ? f.x : pair_value(e0, K);
+        pv[2 * v + 1] = is_escape(e1) ? f.y : pair_value(e1, K);
     }
+    double d = 0.0;
 #pragma unroll
     for (int r = 0; r < RPL; ++r) d = fma(__ldg(B + ((r >> 1) * G + lane) * 2 + (r & 1)), pv[r], d);
     return d;
@@ -341,7 +340,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
     const int qa = (int)min((int64_t)p0 + (int64_t)g * vlen, (int64_t)p1);
     const int qb = min(qa + vlen, p1);
 
-    int K = nm1 * pair_scale(nm1);
+    int K = kPairTop;
     for (int m = 0; m <= nm1; ++m)
         if (m != a.mode) K -= __ldg(a.kexp + m);
     // the FP32 sums carry 2^(K + kDfV), the FP64 accumulator nothing, so that it has the
@@ -494,10 +493,9 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
     auto form_rows = [&](int q) {
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            uint32_t bad = 0;
 #pragma unroll
             for (int v = 0; v < VP; ++v) {
-                PairProduct<true> y0, y1;
+                PairProduct y0, y1;
 #pragma unroll
                 for (int k = 0; k < MAXK; ++k) {
                     if (k < nm1) {
@@ -512,34 +510,9 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
                         }
                     }
                 }
-                const float2 e0 = y0.zero() ? make_float2(0.f, 0.f) : y0.p;
-                const float2 e1 = y1.zero() ? make_float2(0.f, 0.f) : y1.p;
+                const float2 e0 = y0.value(), e1 = y1.value();
                 ph[u][v] = make_float2(e0.x, e1.x);
                 pl[u][v] = make_float2(e0.y, e1.y);
-                bad |= (y0.pair_ok() || y0.zero() ? 0u : 1u) << (2 * v);
-                bad |= (y1.pair_ok() || y1.zero() ? 0u : 1u) << (2 * v + 1);
-            }
-            if (__builtin_expect(bad != 0u, 0)) {
-                // an element below the window for certain needs no value here: an escape
-                // of 0 leaves it out like any small one, and pair_resum forms it where it
-                // matters (with the FP64 product of each, a quarter of all elements along
-                // a solve, launches of the 3-way tensor grew from 0.85 to 4.8 ms in 24 outer
-                // iterations; now to 3.2)
-#pragma unroll
-                for (int r = 0; r < RPL; ++r) {
-                    float &h = r % 2 ? ph[u][r / 2].y : ph[u][r / 2].x;
-                    if (((bad >> r) & 1u) && fabsf(h) < 0.5f * kPairLowF) {
-                        h = __uint_as_float(0x80000000u);
-                        bad &= ~(1u << r);
-                    }
-                }
-#pragma unroll
-                for (int r = 0; r < RPL; ++r)
-                    if ((bad >> r) & 1u) {
-                        const float2 e = pair_exact(a, nm1, K, min(q + u, p1 - 1), col(r / 2) + r % 2);
-                        (r % 2 ? ph[u][r / 2].y : ph[u][r / 2].x) = e.x;
-                        (r % 2 ? pl[u][r / 2].y : pl[u][r / 2].x) = e.y;
-                    }
             }
         }
     };
@@ -568,10 +541,9 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
             for (int v = 0; v < VP; ++v)
                 top_bits = max(top_bits, max(__float_as_uint(ph[u][v].x), __float_as_uint(ph[u][v].y)));
         if (__builtin_expect((int)top_bits < 0, 0)) {
-            // one above the pairs' window (beyond its factor's exponent), or any
-            // where B is not safe, sends its nonzero to FP64
+            // one above the pairs' window, or any where B is not safe, sends its
+            // nonzero to FP64
             const bool unsafe = OP == OP_PHI && !(top < bmax);
-            const uint32_t high = 0x80000000u | ((uint32_t)max(1023 + kPairLow - K, 0) << 20);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 uint32_t e8 = 0, big = 0;
@@ -587,7 +559,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
                 }
                 if (u < m) {
                     em |= e8 << (8 * u);
-                    if (e8 && (unsafe || big >= high)) redo |= 1u << u;
+                    if (e8 && (unsafe || big >= kHighEscape)) redo |= 1u << u;
                 }
             }
         }

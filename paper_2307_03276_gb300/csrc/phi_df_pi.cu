@@ -20,12 +20,12 @@ __global__ void __launch_bounds__(256) factor_max_kernel(const double *__restric
     if ((threadIdx.x & 31) == 0 && m > 0.0) atomicMax(top, ordered_bits(m));
 }
 
-// The pairs of one factor, scaled by 2^(c - k).  top: the largest entry's bits
+// The pairs of one factor, scaled by 2^(kPairTop - k).  top: the largest entry's bits
 // (k is its exponent, held to [-100, 100] so that products' scales stay far
 // inside the FP64 range; entries outside the window escape), or null after a
 // normalisation (entries <= 1: k = 0).  Bound by its 16 bytes per entry.
 __global__ void __launch_bounds__(256) pair_factor_kernel(const double2 *__restrict__ A, float4 *__restrict__ P,
-                                                          int64_t nv, int c,
+                                                          int64_t nv,
                                                           const unsigned long long *__restrict__ top,
                                                           int32_t *__restrict__ kexp) {
     int k = 0;
@@ -36,14 +36,15 @@ __global__ void __launch_bounds__(256) pair_factor_kernel(const double2 *__restr
     if (blockIdx.x == 0 && threadIdx.x == 0) *kexp = k;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nv; e += (int64_t)gridDim.x * blockDim.x) {
         const double2 x = A[e];
-        const float2 p = pair_factor(x.x, c - k, c), q = pair_factor(x.y, c - k, c);
+        const float2 p = pair_factor(x.x, kPairTop - k), q = pair_factor(x.y, kPairTop - k);
         P[e] = make_float4(p.x, q.x, p.y, q.y);
     }
 }
 
 // Khatri-Rao rows of one mode as pairs, like pi_build_range: one thread per
 // 16-byte vector (two elements).  The products are formed as the fused kernel
-// forms them (form_rows in df_walk), so the two give the same bits.
+// forms them (form_rows in df_walk), so the two give the same bits.  No FP64: an
+// element outside the pairs' window is marked, its value left to the few that need it.
 template <int NM1>
 __global__ void __launch_bounds__(256) pi_pair_kernel(const PhiArgs a, float4 *__restrict__ pi) {
     constexpr int MAXK = NM1 > 0 ? NM1 : kMaxNm1;
@@ -51,14 +52,11 @@ __global__ void __launch_bounds__(256) pi_pair_kernel(const PhiArgs a, float4 *_
     const int vpr = a.Rp / 2;  // vectors per row, a power of two
     const int lg = 31 - __clz(vpr);
     const int64_t total = a.nnz << lg;
-    int K = nm1 * pair_scale(nm1);
-    for (int m = 0; m <= nm1; ++m)
-        if (m != a.mode) K -= __ldg(a.kexp + m);
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t p = e >> lg;
         const int v = (int)(e & (vpr - 1));
         int32_t ii[MAXK];
-        PairProduct<false> q0, q1;
+        PairProduct q0, q1;
 #pragma unroll
         for (int k = 0; k < MAXK; ++k) {
             if (k < nm1) {
@@ -73,19 +71,17 @@ __global__ void __launch_bounds__(256) pi_pair_kernel(const PhiArgs a, float4 *_
                 }
             }
         }
-        auto exact = [&](int c) -> float2 {
-            double d = 0.0;
-#pragma unroll
-            for (int k = 0; k < MAXK; ++k)
-                if (k < nm1) {
-                    const double f = __ldg(reinterpret_cast<const double *>(a.A[k]) + (int64_t)ii[k] * a.Rp + c);
-                    d = k == 0 ? f : d * f;
-                }
-            return pair_encode(d, K, kPairMax);
-        };
-        if (!q0.pair_ok()) q0.p = q0.zero() ? make_float2(0.f, 0.f) : exact(2 * v);
-        if (!q1.pair_ok()) q1.p = q1.zero() ? make_float2(0.f, 0.f) : exact(2 * v + 1);
-        __stcs(pi + e, make_float4(q0.p.x, q1.p.x, q0.p.y, q1.p.y));
+        float2 e0 = q0.p, e1 = q1.p;
+        // pairs, then zeros (a padded rank's columns), then the rest; with four gathered
+        // factors both at once (R = 33: 0.502 against 0.514 ms a mode at 3e6 nonzeros; three
+        // factors, R = 16, 2e7: 0.696 against 0.684)
+        const bool plain = NM1 == 4 ? q0.plain() && q1.plain()
+                                    : (q0.pair_ok() && q1.pair_ok()) || (q0.plain_zero() && q1.plain_zero());
+        if (!plain) {
+            e0 = q0.value();
+            e1 = q1.value();
+        }
+        __stcs(pi + e, make_float4(e0.x, e1.x, e0.y, e1.y));
     }
 }
 
@@ -135,8 +131,7 @@ cpapr_status launch_factor_pairs(cpapr_ctx *ctx, int m, bool from_data) {
         CPAPR_CUDA(ctx, cudaGetLastError());
     }
     pair_factor_kernel<<<grid, 256, 0, ctx->stream>>>(reinterpret_cast<const double2 *>(A),
-                                                      reinterpret_cast<float4 *>(ctx->P[m]), n / 2,
-                                                      pair_scale(ctx->N - 1), top, ctx->kexp + m);
+                                                      reinterpret_cast<float4 *>(ctx->P[m]), n / 2, top, ctx->kexp + m);
     CPAPR_CUDA(ctx, cudaGetLastError());
     count_launch(ctx, from_data ? 2 : 1);
     return CPAPR_OK;
