@@ -103,8 +103,11 @@ enum { CPAPR_DOT_AUTO = 0, CPAPR_DOT_FP64 = 1, CPAPR_DOT_FP32_PIPE = 2 };
  *             evaluated in FP64.  CPAPR_DOT_AUTO (default): the FP32 pipe where
  *             the tensor has at least 608 tiles (4 per SM; of 2048 nonzeros, 1024
  *             from rank 17 on, or of tile_nnz), FP64 below that, where one tile's
- *             latency bounds the launch.  The batched solver always takes
- *             FP64.  Ignored in FP32.
+ *             latency bounds the launch; and rows and scaled addition in FP64
+ *             again, only the dot and the division on the FP32 pipe, in modes
+ *             where the model's entries have decayed so far that this is faster
+ *             (looked at once per outer iteration, from the factors alone).  The
+ *             batched solver always takes FP64.  Ignored in FP32.
  *  tune_cache NULL (default) or the path of a text file of tuned choices,
  *             one line per shape class: precision, number of modes, padded
  *             rank, and power-of-two buckets of the nonzeros, of the mode's
@@ -323,7 +326,7 @@ typedef struct {
     int32_t precision;
     int64_t nnz;
     int64_t dims[CPAPR_MAX_MODES];
-    int32_t tile_nnz[CPAPR_MAX_MODES];    /* chosen per mode (of its Phi launches) */
+    int32_t tile_nnz[CPAPR_MAX_MODES];    /* chosen per mode (of its Phi launches, as of the last one) */
     int32_t rank_lanes[CPAPR_MAX_MODES];  /* chosen per mode */
     int32_t reduction[CPAPR_MAX_MODES];   /* chosen per mode */
     int32_t ntiles[CPAPR_MAX_MODES];

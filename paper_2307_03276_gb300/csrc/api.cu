@@ -631,7 +631,7 @@ cpapr_status cpapr_set_model(cpapr_ctx *ctx, const double *lambda, const double 
     if (flags[0]) return fail(ctx, CPAPR_E_VALUE, "lambda must be finite and >= 0");
     ctx->k_total = 0;
     ctx->pi_mode_built = -1;
-    for (int m = 0; m < ctx->N; ++m) ctx->pair_state[m] = kPairStale;
+    for (int m = 0; m < ctx->N; ++m) factor_changed(ctx, m, kPairStale);
     if (flags[2]) {
         ctx->model_set = false;
         return fail(ctx, CPAPR_E_VALUE, "factor entries must be finite and >= 0");
@@ -643,7 +643,7 @@ cpapr_status cpapr_set_model(cpapr_ctx *ctx, const double *lambda, const double 
 cpapr_status cpapr_init_random(cpapr_ctx *ctx, uint64_t seed) {
     API_ENTER(ctx);
     CPAPR_TRY(launch_init_random(ctx, seed));
-    for (int m = 0; m < ctx->N; ++m) ctx->pair_state[m] = kPairStale;
+    for (int m = 0; m < ctx->N; ++m) factor_changed(ctx, m, kPairStale);
     for (int m = 0; m < ctx->N; ++m)
         CPAPR_CUDA(ctx, cudaMemsetAsync(ctx->Phi[m], 0, (size_t)ctx->dims[m] * ctx->Rp * ctx->esize, ctx->stream));
     CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
@@ -712,7 +712,7 @@ cpapr_status cpapr_set_state(cpapr_ctx *ctx, const double *lambda, const double 
     // after an outer iteration every factor is normalised: the pairs' exponents are
     // those of the solve that goes on, not measured again (as for a model just set)
     if (outer_done > 0)
-        for (int m = 0; m < ctx->N; ++m) ctx->pair_state[m] = kPairNormalised;
+        for (int m = 0; m < ctx->N; ++m) factor_changed(ctx, m, kPairNormalised);
     return CPAPR_OK;
 }
 
@@ -756,6 +756,7 @@ cpapr_status cpapr_phi(cpapr_ctx *ctx, int32_t mode, const double *B, double *ou
     }
     // Phi[mode] holds the previous iteration's Phi that S reads: compute into
     // the separate output buffer instead.
+    CPAPR_TRY(ensure_routes(ctx, 1u << mode));
     CPAPR_TRY(prepare_phi(ctx, mode));
     CPAPR_TRY(launch_phi(ctx, mode, OP_PHI, ctx->B, ctx->outbuf, nullptr));
     CPAPR_TRY(download_matrix(ctx, ctx->outbuf, ctx->dims[mode], out));

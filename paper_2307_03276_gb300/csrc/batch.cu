@@ -629,7 +629,7 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
     for (int i = 0; i < count; ++i) {
         CPAPR_CUDA(ctxs[i], cudaStreamSynchronize(ctxs[i]->stream));
         ctxs[i]->pi_mode_built = -1;  // the batched solve changes every factor
-        for (int m = 0; m < N; ++m) ctxs[i]->pair_state[m] = kPairStale;
+        for (int m = 0; m < N; ++m) factor_changed(ctxs[i], m, kPairStale);
     }
     // every tensor needs a rank class of the batched kernel and the segmented
     // reduction; it keeps its own tile size (tuned or heuristic) as long as
@@ -766,7 +766,7 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
             a.llpart = c->llpart;
             a.err = c->errflag + 3;
             a.stage_extra = injected_stage_shortfall();
-            a.dfdot = 0;  // the batched kernel keeps FP64 rows and the FP64 dot
+            a.route = kRouteFp64;  // the batched kernel keeps FP64 rows and the FP64 dot
             // FP64 tensors whose mode n materialises its Khatri-Rao rows stream them here too
             if (sizeof(T) == 8 && L.pi && c->pibuf && c->nnz > 0) {
                 a.pi = c->pibuf;

@@ -78,16 +78,6 @@ __device__ __forceinline__ void df_cut(double x, int s, float &hi, float &lo) {
     }
 }
 
-// a + b for hi/lo float pairs with |lo| <= ulp(hi) / 2 (Knuth's two-sum of the
-// highs, then a fast two-sum that renormalises); the result is such a pair
-__device__ __forceinline__ float2 df_add(float2 a, float2 b) {
-    const float s = a.x + b.x;
-    const float z = s - a.x;
-    const float e = ((a.x - (s - z)) + (b.x - z)) + (a.y + b.y);
-    const float h = s + e;
-    return make_float2(h, e - (h - s));
-}
-
 // S + C += a b for pairs a, b >= 0, two columns at once (.x and .y: Blackwell's
 // packed FP32 instructions take two per lane and issue slot; the kernel is bound by
 // issue).  t = S + a_hi b_hi is rounded once (FMA); its error is (S - (t - z)) +
@@ -149,30 +139,6 @@ __device__ __forceinline__ bool df_bad_x(double x) {
     const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
     const unsigned e = (unsigned)(bits >> 52);
     return bits != 0ull && (e < 1023u - 20u || e >= 1023u + 30u);
-}
-
-// the reduce-scatter of group_reduce_scatter for pairs, over the whole warp
-template <int G, int U>
-__device__ __forceinline__ float2 group_reduce_scatter_df(float2 (&s)[U], int lane) {
-    static_assert(U <= G, "reduce-scatter needs U <= G");
-    constexpr unsigned full = 0xffffffffu;
-    int o = G / 2;
-#pragma unroll
-    for (int h = U / 2; h >= 1; h >>= 1) {
-        const bool upper = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < h; ++i) {
-            const float2 send = upper ? s[i] : s[i + h];
-            const float2 keep = upper ? s[i + h] : s[i];
-            s[i] = df_add(keep, make_float2(__shfl_xor_sync(full, send.x, o), __shfl_xor_sync(full, send.y, o)));
-        }
-        o >>= 1;
-    }
-    float2 tot = s[0];
-#pragma unroll
-    for (int oo = G / (2 * U); oo > 0; oo >>= 1)
-        tot = df_add(tot, make_float2(__shfl_xor_sync(full, tot.x, oo), __shfl_xor_sync(full, tot.y, oo)));
-    return tot;
 }
 
 // (The paths that are rarely taken are inlined all the same: as called functions
@@ -602,7 +568,7 @@ __global__ void __launch_bounds__(kDfThreads, kDfBlocks) phi_pair_kernel(const _
                 if (OP == OP_LL && u < m && !((redo >> u) & 1u)) ll += x[G > 1 ? 0 : u] * log(m_ll);
             }
         } else {
-            const float2 tot = group_reduce_scatter_df<G, U>(s2, lane);
+            const float2 tot = group_reduce_scatter_df<G, U>(s2, lane, full);
             if (OP == OP_LL && __builtin_expect(__any_sync(full, em != 0u), 0)) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) drop_ok(__shfl_sync(full, tot.x, gbase + u * LPU), u);

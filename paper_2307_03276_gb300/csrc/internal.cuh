@@ -54,6 +54,7 @@ struct HostSlot {
     InnerState inner[kMaxModes];
     double ll;
     int32_t flags[4];
+    int32_t resum[kMaxModes][2];  // the route probe's counts
 };
 HostSlot *host_slot_acquire();  // null if none can be had
 void host_slot_release(HostSlot *s);
@@ -77,6 +78,7 @@ struct ModeLayout {
     // a launch takes 2^k of these tiles as one (heuristic_config): k = sh, sh_df for
     // the kernels over float pairs, batch_sh in the batched solver
     int32_t sh = 0, sh_df = 0, batch_sh = 0;
+    bool late = false;             // the float pairs are slower than the FP64 rows by now (route.cu)
     int32_t pi = 0;                // 1: Phi streams the materialised Khatri-Rao rows (built per outer iteration)
     int32_t nempty = 0;
     int32_t *erows = nullptr;      // [nempty] rows without nonzeros, increasing
@@ -107,11 +109,13 @@ struct cpapr_ctx {
     size_t factor_bytes = 0;
     cudaAccessPolicyWindow l2win{};  // persisting-L2 window over factor_block (num_bytes 0: none)
     void *B = nullptr;
-    // FP64 form, where a mode's Phi runs on float pairs (uses_pairs): the
+    // FP64 form, where a mode's Phi may run on float pairs (phi_route): the
     // factors as pairs, their exponents, and which copies are current
     float2 *P[CPAPR_MAX_MODES] = {};
     int32_t *kexp = nullptr;                    // [N]
     unsigned long long *pair_top = nullptr;     // [N] largest entries (scratch of launch_factor_pairs)
+    int32_t *resum = nullptr;                   // [N][2] counts of the route probe
+    uint32_t routes_known = 0;                  // modes whose `late` is the current factors'
     int pair_state[CPAPR_MAX_MODES] = {};       // kPairStale, kPairNormalised (stale, entries <= 1) or kPairCurrent
     // FP32 form: FP64 masters of the factors and of B.  The multiplicative
     // update, the shift S and the normalisation run on them in FP64 and
@@ -127,6 +131,7 @@ struct cpapr_ctx {
     int64_t carry_elems = 0;
     void *pibuf = nullptr;  // materialised Khatri-Rao rows of the current mode [nnz_pad x Rp]
     int pi_mode_built = -1;  // mode whose rows pibuf holds, built from the current other factors (-1: none)
+    bool pi_pairs = false;   // pibuf holds them as float pairs
     int64_t llpart_n = 0;    // capacity of llpart (tiles)
     double *colpart = nullptr;   // column-sum partials [N x kColParts x Rp]
     unsigned int *llcount = nullptr;  // last-block counters (zero between launches): [0] log-likelihood total, [1] normalisation column sums
@@ -153,6 +158,7 @@ struct cpapr_ctx {
     // graphs (one per mode and inner-loop bound)
     cudaGraphExec_t graph_exec[CPAPR_MAX_MODES] = {};
     int graph_max_inner[CPAPR_MAX_MODES] = {};
+    int graph_route[CPAPR_MAX_MODES] = {};
     double graph_tol[CPAPR_MAX_MODES] = {};
 };
 
@@ -160,7 +166,7 @@ namespace cpapr {
 
 constexpr int kColParts = 256;
 enum { kPairStale = 0, kPairNormalised = 1, kPairCurrent = 2 };
-// tiles from which an FP64 Phi launch takes the kernel with its dot on the FP32 pipe
+// tiles from which an FP64 Phi launch leaves the FP64 pipe (phi_route)
 constexpr int kDfMinTiles = 152 * 4;
 // below this many tiles the automatic tile size shrinks (heuristic_config)
 constexpr int kSmallTiles = 152 * 4;
@@ -223,8 +229,23 @@ enum PhiOp { OP_PHI = 0, OP_MTTKRP = 1, OP_LL = 2 };
 // B: I_n x Rp of the working type (ignored for MTTKRP).  inner: state whose
 // done flag / kkt slot the kernels use (may be null for a one-off Phi).
 cpapr_status launch_phi(cpapr_ctx *ctx, int n, PhiOp op, const void *B, void *out, InnerState *inner);
-// does Phi of mode n run on float pairs (df_pair.cuh)?
-bool uses_pairs(const cpapr_ctx *ctx, int n);
+// how Phi of mode n runs: FP64; FP64 rows with the divisor on the FP32 pipe
+// (phi_kernels.cuh); on float pairs (df_walk.cuh).  FP32 contexts: kRouteFp64.
+enum PhiRoute { kRouteFp64 = 0, kRoutePipe = 1, kRoutePairs = 2 };
+PhiRoute phi_route(const cpapr_ctx *ctx, int n);
+inline bool uses_pairs(const cpapr_ctx *ctx, int n) { return phi_route(ctx, n) == kRoutePairs; }
+// is that a choice the factors decide (route.cu)?
+bool route_varies(const cpapr_ctx *ctx, int n);
+// factor m is no longer what its pairs and the routes were made from
+inline void factor_changed(cpapr_ctx *ctx, int m, int state) {
+    ctx->pair_state[m] = state;
+    ctx->routes_known = 0;
+}
+// the routes of the modes in the mask from the current factors: the probe and its
+// copy to the host queued; taken up after a synchronisation; both at once
+cpapr_status queue_routes(cpapr_ctx *ctx, uint32_t modes);
+void take_routes(cpapr_ctx *ctx, uint32_t modes);
+cpapr_status ensure_routes(cpapr_ctx *ctx, uint32_t modes);
 // log2 of the table tiles per tile of mode n's Phi launch
 inline int phi_shift(const cpapr_ctx *ctx, int n) {
     return uses_pairs(ctx, n) ? ctx->mode[n].sh_df : ctx->mode[n].sh;

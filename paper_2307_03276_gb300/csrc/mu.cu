@@ -233,7 +233,7 @@ cpapr_status launch_normalise(cpapr_ctx *ctx, int n) {
     const int parts = colsum_parts(rows, Rp);
     // A^(n) changes: materialised rows of another mode that contain it go stale
     if (n != ctx->pi_mode_built) ctx->pi_mode_built = -1;
-    ctx->pair_state[n] = kPairNormalised;
+    factor_changed(ctx, n, kPairNormalised);
     ProfScope ps(ctx, K_NORM);
     count_launch(ctx, 2);
     // llcount[1]: the column-sum counter (llcount[0] belongs to the log-likelihood total)
@@ -556,7 +556,7 @@ cpapr_status upload_matrix(cpapr_ctx *ctx, const double *src, int64_t rows, void
 }
 
 cpapr_status upload_factor(cpapr_ctx *ctx, int m, const double *src) {
-    ctx->pair_state[m] = kPairStale;
+    factor_changed(ctx, m, kPairStale);
     return upload_matrix2(ctx, src, ctx->dims[m], ctx->A[m], ctx->A64[m]);
 }
 

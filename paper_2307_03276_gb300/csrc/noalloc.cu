@@ -89,6 +89,10 @@ extern "C" cpapr_status cpapr_phi_noalloc(cpapr_ctx *ctx, int32_t mode, const do
     if (!out || !is_device_pointer(out)) return fail(ctx, CPAPR_E_ARG, "out must be a device pointer");
     if (B && !is_device_pointer(B)) return fail(ctx, CPAPR_E_ARG, "B must be NULL or a device pointer");
     const ModeLayout &L = ctx->mode[mode];
+    DeviceGuard guard(ctx->device);
+    if (guard.err != cudaSuccess)
+        return fail(ctx, CPAPR_E_CUDA, std::string("selecting the context's device: ") + cudaGetErrorString(guard.err));
+    CPAPR_TRY(ensure_routes(ctx, 1u << mode));
     // cpapr_phi's tiles, or those of the mode's other launches where only these fit the
     // scratch (padded rank 128 over float pairs: 512 nonzeros, and 1024)
     int sh = phi_shift(ctx, mode);
@@ -104,9 +108,6 @@ extern "C" cpapr_status cpapr_phi_noalloc(cpapr_ctx *ctx, int32_t mode, const do
                         std::to_string(tiles) + " tiles x " + std::to_string(ctx->Rp) +
                         " ranks); the fixed scratch holds " + std::to_string((long long)CPAPR_NOALLOC_SCRATCH_BYTES) +
                         ": use cpapr_phi, or a larger tile_nnz");
-    DeviceGuard guard(ctx->device);
-    if (guard.err != cudaSuccess)
-        return fail(ctx, CPAPR_E_CUDA, std::string("selecting the context's device: ") + cudaGetErrorString(guard.err));
     void *scratch = nullptr;
     CPAPR_TRY(scratch_address(ctx, &scratch));
     if (ctx->nnz == 0) {

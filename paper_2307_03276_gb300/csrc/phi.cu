@@ -57,8 +57,8 @@ static cudaError_t dispatch(const cpapr_ctx *ctx, const PhiArgs &a, int rpl, int
     const int nm1 = ctx->N - 1;
     // Phi over materialised rows gathers no factor rows: no window
     const cudaAccessPolicyWindow *win = (op == OP_PHI && a.pi) ? nullptr : l2_window(ctx);
-    if (a.dfdot && a.pi && op != OP_MTTKRP) return launch_phi_df_pi(a, op, ctx->stream, win);
-    if (a.dfdot && op == OP_PHI) {
+    if (a.route == kRoutePairs && a.pi && op != OP_MTTKRP) return launch_phi_df_pi(a, op, ctx->stream, win);
+    if (a.route == kRoutePairs && op == OP_PHI) {
         switch (nm1) {
             case 2: return launch_phi_df_n2(a, ctx->stream, win);
             case 3: return launch_phi_df_n3(a, ctx->stream, win);
@@ -101,21 +101,31 @@ uint32_t injected_stage_shortfall() {
     return (s && s[0] == '1' && s[1] == 0) ? 16u : 0u;
 }
 
-// FP64 Phi on float pairs: accurate relative to max(s, eps) for the eps its
+// Off the FP64 pipe an FP64 Phi is accurate relative to max(s, eps) for the eps its
 // scales cover, and faster where the launch has at least a wave of tiles (4 per
 // SM); a launch of a few tiles is bound by one tile's latency, which the longer
 // FP32 instruction chains raise.
-static bool pairs_apply(const cpapr_ctx *ctx, int n) {
+static bool off_fp64_pipe(const cpapr_ctx *ctx, int n) {
     const ModeLayout &L = ctx->mode[n];
     const int dot = ctx->opt.fp64_dot;
     if (L.tile_nnz == 0) return false;  // not configured yet
     return ctx->esize == 8 && ctx->nnz > 0 && ctx->Rp / L.lanes <= 8 && ctx->opt.eps >= 0x1p-43 &&
-           ctx->opt.eps <= 0x1p20 &&
+           ctx->opt.eps < 0x1p31 &&
            (dot == CPAPR_DOT_FP32_PIPE ||
             (dot == CPAPR_DOT_AUTO && ceil_div(ctx->nnz, (int64_t)L.tile_nnz << L.sh) >= kDfMinTiles));
 }
 
-bool uses_pairs(const cpapr_ctx *ctx, int n) { return ctx->P[0] && pairs_apply(ctx, n); }
+static bool pairs_apply(const cpapr_ctx *ctx, int n) { return off_fp64_pipe(ctx, n) && ctx->opt.eps <= 0x1p20; }
+
+bool route_varies(const cpapr_ctx *ctx, int n) {
+    return ctx->P[0] && ctx->opt.fp64_dot == CPAPR_DOT_AUTO && pairs_apply(ctx, n);
+}
+
+PhiRoute phi_route(const cpapr_ctx *ctx, int n) {
+    if (!off_fp64_pipe(ctx, n)) return kRouteFp64;
+    if (!ctx->P[0] || !pairs_apply(ctx, n)) return kRoutePipe;
+    return ctx->mode[n].late && ctx->opt.fp64_dot == CPAPR_DOT_AUTO ? kRoutePipe : kRoutePairs;
+}
 
 // The factors as pairs, where some mode's Phi would read them.  A context without
 // the room for them (8 bytes per padded factor entry) keeps the kernels that need none.
@@ -135,6 +145,7 @@ cpapr_status ensure_pair_storage(cpapr_ctx *ctx) {
     char *base = (char *)p;
     ctx->pair_top = (unsigned long long *)(base + ofs[ctx->N]);
     ctx->kexp = (int32_t *)(base + ofs[ctx->N] + 128);
+    ctx->resum = (int32_t *)(base + ofs[ctx->N] + 192);
     for (int m = 0; m < ctx->N; ++m) {
         ctx->P[m] = (float2 *)(base + ofs[m]);
         ctx->pair_state[m] = kPairStale;
@@ -184,7 +195,7 @@ static PhiArgs make_args(cpapr_ctx *ctx, int n, const void *B, void *out, InnerS
     a.llpart = ctx->llpart;
     a.err = ctx->errflag + 3;
     a.stage_extra = injected_stage_shortfall();
-    a.dfdot = uses_pairs(ctx, n) ? 1 : 0;
+    a.route = phi_route(ctx, n);
     a.mode = n;
     a.kexp = ctx->kexp;
     for (int m = 0, j = 0; m < ctx->N; ++m)
@@ -277,11 +288,12 @@ cpapr_status prepare_phi(cpapr_ctx *ctx, int n) {
     PhiArgs a = make_args(ctx, n, nullptr, nullptr, nullptr);
     ProfScope ps(ctx, K_PI);
     count_launch(ctx);
-    const cudaError_t e = a.dfdot           ? launch_pi_pairs(a, ctx->pibuf, ctx->stream, l2_window(ctx))
+    const cudaError_t e = a.route == kRoutePairs ? launch_pi_pairs(a, ctx->pibuf, ctx->stream, l2_window(ctx))
                           : ctx->esize == 8 ? run_pi_build<double>(a, (double *)ctx->pibuf, ctx->stream, l2_window(ctx))
                                             : run_pi_build<float>(a, (float *)ctx->pibuf, ctx->stream, l2_window(ctx));
     if (e != cudaSuccess) return cuda_fail(ctx, e, "Pi build kernel");
     ctx->pi_mode_built = n;
+    ctx->pi_pairs = a.route == kRoutePairs;
     return CPAPR_OK;
 }
 
@@ -351,8 +363,10 @@ cpapr_status launch_loglik(cpapr_ctx *ctx, double *dst) {
     PhiArgs a = make_args(ctx, n, ctx->B, nullptr, nullptr);
     a.atomic = 0;
     if (use_pi) {
+        // (the mode's route may have changed since they were built)
         a.pi = ctx->pibuf;
-        set_tiles(a, L, phi_shift(ctx, n));
+        a.route = ctx->pi_pairs ? kRoutePairs : kRouteFp64;
+        set_tiles(a, L, ctx->pi_pairs ? L.sh_df : L.sh);
     }
     {
         ProfScope ps(ctx, K_LL);

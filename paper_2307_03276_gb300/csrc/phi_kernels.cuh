@@ -38,7 +38,8 @@
 //
 // Which launches run this kernel: FP64 Phi below a wave of tiles, FP64 MTTKRP,
 // the fused log-likelihood and 3-way FP32 MTTKRP.  Large FP64 Phi launches work on
-// float pairs (df_walk.cuh) and the other FP32 launches in direct.cuh; both share
+// float pairs (df_walk.cuh), or here with the dot on the FP32 pipe once a model's
+// entries have left the pairs' window (route.cu), and the other FP32 launches in direct.cuh; both share
 // the three levels above (segmented_tail) and the violation.
 //
 // FP32 form: gathers, Khatri-Rao products, dot and scale in FP32; a run of
@@ -93,9 +94,9 @@ struct PhiArgs {
     // log-likelihood reads where an FP32 model value underflows (else null)
     const double *Bm;
     const double *Am[kMaxNm1];
-    // FP64 Phi on the FP32 pipe (dfdot = 1): the gathered factors as float pairs
-    // and their exponents k_m (kexp[m], m = 0..nm1; `mode` is the one not gathered)
-    int32_t dfdot;
+    // FP64 Phi (PhiRoute): on float pairs, the gathered factors as pairs and their
+    // exponents k_m (kexp[m], m = 0..nm1; `mode` is the one not gathered)
+    int32_t route;
     int32_t mode;
     const float2 *P[kMaxNm1];
     const int32_t *kexp;
@@ -185,6 +186,139 @@ __device__ __forceinline__ double phi_divide(double x, double s, double eps) {
     return x * r;
 }
 __device__ __forceinline__ float phi_divide(float x, float s, float eps) { return __fdividef(x, s > eps ? s : eps); }
+
+// ---- the FP64 form's dot product on the FP32 pipe ---------------------------------
+//
+// GB300 issues 64 FP32 FMAs for every FP64 FMA.  In the FP64 Phi kernel the dot
+// s = <B[i_n], pi> is the divisor of x and only has to be accurate relative to
+// max(s, eps), so it runs on the FP32 pipe: each FP64 operand is cut into two
+// floats hi + lo holding its leading 48 significant bits (integer operations),
+// each product hi_a hi_b is taken exactly with an FMA (Dekker's product p + e),
+// the products p are added with Knuth's two-sum (the rounding error of every
+// addition is kept), and the errors e, the cross products hi_a lo_b + lo_a hi_b
+// and the two-sum errors are summed in plain FP32.  For k terms, all >= 0,
+// with u = 2^-24 (first order):
+//   operands cut to 48 bits:                 <= 2.5 * 2^-47 s
+//   e and cross terms (3k sums of terms <= 3u s):  <= 9k u^2 s
+//   two-sum errors (k sums of terms <= u s):        <= k^2 u^2 s
+//   operands below 2^-126 dropped:           < k 2^31 2^-126 (absolute)
+// For k = 8 ranks per lane: |s_df - s| <= 5.2e-13 s + 2^-92, i.e. below 6e-13
+// relative to max(s, eps) for eps >= 2^-43.  The lanes' partials are added
+// as hi/lo pairs (df_add) and x / max(s, eps) is taken on the FP32 pipe as well
+// (df_divide, within 2^-43 relative), so v = x / max(s, eps) is within 7.5e-13
+// relative, inside the FP64 form's 1e-12 parity bound (Phi inherits the
+// relative error of its v, its terms being >= 0); the batch's FP64 operations
+// are one addition per division and the scale-add.  An operand >= 2^31
+// (beyond the exponents the cut assumes) or a value x outside {0} and
+// [2^-20, 2^31) makes the group redo the batch with the FP64 dot and division.
+
+// x >= 0 as hi + lo, its leading 48 significant bits (integer operations and
+// one integer-to-float conversion); x < 2^-126 gives 0 + 0, x >= 2^31 sets big.
+__device__ __forceinline__ void df_cut(double x, float &hi, float &lo, bool &big) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    const uint32_t H = (uint32_t)(bits >> 32), L = (uint32_t)bits;
+    const int e = (int)(H >> 20);  // biased exponent (x >= 0)
+    big = big || e >= 1023 + 31;
+    const bool keep = e >= 1023 - 126;
+    // hi: the first 23 fraction bits with the exponent rebased from bias 1023
+    // to bias 127 (896 less in the exponent field)
+    hi = keep ? __uint_as_float(__funnelshift_l(L, H, 3) - (896u << 23)) : 0.f;
+    // lo: the next 29 fraction bits (24 kept) times 2^(e - 1075), scaled in
+    // two exact steps that stay in the float range
+    const float m = __uint2float_rz(L & 0x1fffffffu);
+    lo = keep ? m * __uint_as_float((uint32_t)(e - 1075 + 64 + 127) << 23) * 0x1p-64f : 0.f;
+}
+
+// a + b for hi/lo float pairs with |lo| <= ulp(hi) / 2 (Knuth's two-sum of the
+// highs, then a fast two-sum that renormalises); the result is such a pair
+__device__ __forceinline__ float2 df_add(float2 a, float2 b) {
+    const float s = a.x + b.x;
+    const float z = s - a.x;
+    const float e = ((a.x - (s - z)) + (b.x - z)) + (a.y + b.y);
+    const float h = s + e;
+    return make_float2(h, e - (h - s));
+}
+
+// sum_r a_r b_r with a given as hi/lo floats (cut once per B row) and b in
+// FP64, as a renormalised hi/lo float pair
+template <int K>
+__device__ __forceinline__ float2 df_dot(const float (&ahi)[K], const float (&alo)[K], const double (&b)[K],
+                                         bool &big) {
+    float S = 0.f, C = 0.f, D = 0.f;
+#pragma unroll
+    for (int r = 0; r < K; ++r) {
+        float bh, bl;
+        df_cut(b[r], bh, bl, big);
+        const float p = __fmul_rn(ahi[r], bh);  // not to be fused into S + p below
+        D = fmaf(ahi[r], bh, -p) + D;
+        D = fmaf(ahi[r], bl, D);
+        D = fmaf(alo[r], bh, D);
+        const float t = S + p;
+        const float z = t - S;
+        C += (S - (t - z)) + (p - z);
+        S = t;
+    }
+    const float E = C + D;
+    const float h = S + E;  // |E| << S: fast two-sum
+    return make_float2(h, E - (h - S));
+}
+
+// x / max(s, eps) in FP64 from the pair s = s.x + s.y and eps = eh + el, on the
+// FP32 pipe: q0 = x_hi / m_hi to single precision (the hardware reciprocal
+// estimate), then the classical correction of a double-length division
+// (Dekker): the residual x - q0 m, formed exactly to first order with the FMA
+// product q0 m_hi = p + pe (x_hi - p is exact: p is within a factor of two of
+// x_hi), divided by m_hi gives q1, and q0 + q1 is the quotient.  |q1| <= 2^-21
+// q0 and q1 carries a relative error of about 2^-22 (estimate, rounding), so
+// the quotient is within 2^-43 relative; x enters with its 48 leading bits
+// (2^-48).  One FP64 addition widens it.  Needs x = 0 or 2^-20 <= x < 2^31
+// (checked by df_check_x), eps >= 2^-43 and s < 2^66 (eight operands < 2^31 per
+// lane, up to 16 lanes), so that q0 and q1 are normal floats.
+__device__ __forceinline__ double df_divide(double x, float2 s, float eh, float el) {
+    float xh, xl;
+    bool unused = false;
+    df_cut(x, xh, xl, unused);
+    const bool use_s = (s.x - eh) + (s.y - el) >= 0.f;  // s.x - eh is exact where they are close
+    const float mh = use_s ? s.x : eh, ml = use_s ? s.y : el;
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(mh));
+    const float q0 = xh * r;
+    const float p = __fmul_rn(q0, mh);
+    const float pe = fmaf(q0, mh, -p);
+    const float res = ((xh - p) - pe) + fmaf(-q0, ml, xl);
+    return df_widen(q0) + df_widen(res * r);
+}
+
+// sets big unless x = 0 or 2^-20 <= x < 2^31 (the range df_divide handles);
+// integer operations on the bits of x >= 0
+__device__ __forceinline__ void df_check_x(double x, bool &big) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+    const unsigned e = (unsigned)(bits >> 52);
+    big = big || (bits != 0ull && (e < 1023u - 20u || e >= 1023u + 31u));
+}
+
+// the reduce-scatter below for hi/lo float pairs (two shuffles per pair)
+template <int G, int U>
+__device__ __forceinline__ float2 group_reduce_scatter_df(float2 (&s)[U], int lane, unsigned gmask) {
+    static_assert(U <= G, "reduce-scatter needs U <= G");
+    int o = G / 2;
+#pragma unroll
+    for (int h = U / 2; h >= 1; h >>= 1) {
+        const bool upper = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float2 send = upper ? s[i] : s[i + h];
+            const float2 keep = upper ? s[i + h] : s[i];
+            s[i] = df_add(keep, make_float2(__shfl_xor_sync(gmask, send.x, o), __shfl_xor_sync(gmask, send.y, o)));
+        }
+        o >>= 1;
+    }
+    float2 tot = s[0];
+#pragma unroll
+    for (int oo = G / (2 * U); oo > 0; oo >>= 1)
+        tot = df_add(tot, make_float2(__shfl_xor_sync(gmask, tot.x, oo), __shfl_xor_sync(gmask, tot.y, oo)));
+    return tot;
+}
 
 // On entry each of the G lanes of a group holds U partial dot products (its
 // RPL ranks) of the group's U nonzeros.  A reduce-scatter halves the set at
@@ -641,7 +775,8 @@ __device__ __forceinline__ void segmented_tail(const PhiArgs &a, const int t, T 
 // PI: the Khatri-Rao rows are read from the materialised Pi (a.pi, one row
 // per nonzero in mode-n order) instead of being formed from the factors; the
 // stage then holds only the row ids and the values.
-template <typename T, int NM1, int RPL, int G, int OP, int THREADS, int U, bool PI = false>
+// DF: the FP64 Phi (8 or fewer ranks per lane) takes its dot on the FP32 pipe.
+template <typename T, int NM1, int RPL, int G, int OP, int THREADS, int U, bool PI = false, bool DF = false>
 __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, unsigned char *smem_raw, double *red,
                                               uint64_t *bar, uint32_t &phase) {
     static_assert(U == 1 || U == 2 || U == 4, "batches of 1, 2 or 4 nonzeros");
@@ -653,9 +788,19 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
     // the tile's first and last row in nzrow, read first so that their latency
     // passes while the block checks its state and synchronises
     int32_t k0 = 0, k1 = 0;
+    // FP64 Phi on the FP32 pipe: the KKT maximum published so far (both slots
+    // and the iteration index, read at once), which seeds the running maximum
+    constexpr bool KSEED = DF && sizeof(T) == 8 && OP == OP_PHI;
+    unsigned long long kslot0 = 0ull, kslot1 = 0ull;
+    int32_t kl = 0;
     if (threadIdx.x == 0) {
         k0 = __ldg(a.krow + ((int64_t)t << a.ksh));
         k1 = __ldg(a.krow + min((int64_t)(t + 1) << a.ksh, (int64_t)a.ntab));
+        if (KSEED && a.inner) {
+            kl = *((volatile int32_t *)&a.inner->l);
+            kslot0 = *((volatile unsigned long long *)&a.inner->kkt[0]);
+            kslot1 = *((volatile unsigned long long *)&a.inner->kkt[1]);
+        }
     }
     if (a.inner && a.inner->done) return true;
     const int nm1 = PI ? 0 : (NM1 > 0 ? NM1 : a.nm1);  // staged coordinate streams
@@ -679,7 +824,8 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
     T *slot_val = reinterpret_cast<T *>(s_cnt + W);                 // [2 * NG][Rp]
     int32_t *slot_row = reinterpret_cast<int32_t *>(slot_val + 2 * NG * Rp);  // [2 * NG]
     int32_t *slot_fin = slot_row + 2 * NG;  // [2]: rows spanning tiles this block finishes
-    int32_t *s_meta = slot_fin + 2;         // [2]: s_rows index of the tile's first row; rows after it
+    int32_t *s_meta = slot_fin + 2;         // [2]: s_rows index of the tile's first row; rows after it;
+                                            // then 8 bytes: the KKT maximum published so far
     // the staged bits start at the 16-byte group holding bit p0 and run
     // through the word holding bit p1 (whether the last row goes on)
     const int64_t w0 = (p0 >> 5) & ~(int64_t)3;
@@ -704,6 +850,8 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
         stage_copy(s_rows, a.nzrow + k0a, br, bar);
         s_meta[0] = k0 - k0a;
         s_meta[1] = k1 - k0;
+        // the maximum published so far: terms below it cannot change the result
+        if constexpr (KSEED) *reinterpret_cast<unsigned long long *>(s_meta + 2) = (kl & 1) ? kslot1 : kslot0;
     }
     const bool segmented = (OP != OP_LL) && !a.atomic;
     if (segmented) {
@@ -750,6 +898,11 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
     const T *__restrict__ Bm = reinterpret_cast<const T *>(a.B);
     T *__restrict__ out = reinterpret_cast<T *>(a.out);
     const T eps = (T)a.eps;
+    float eps_hi = 0.f, eps_lo = 0.f;  // eps as a hi/lo float pair (FP32-pipe division)
+    {
+        bool unused = false;
+        df_cut(a.eps, eps_hi, eps_lo, unused);
+    }
 
     // Contiguous run [la, lb) of the tile for this group.  Runs start on
     // multiples of U (vector loads of a batch).  With one lane per group an
@@ -764,7 +917,9 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
     }
     const int la = min(g * vlen, n), lb = min(la + vlen, n);
 
+    // running KKT maximum, from the one published so far (FP64 Phi on the FP32 pipe)
     T kkt = T(0);
+    if constexpr (KSEED) kkt = (T)__longlong_as_double(*reinterpret_cast<const long long *>(s_meta + 2));
     double ll = 0.0;
     // with G > 1 lanes each lane finishes one nonzero of the batch: u_mine
     constexpr int LPU = G > 1 ? G / U : 1;  // lanes per nonzero after the reduce-scatter
@@ -774,7 +929,12 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
     // lanes, whose registers go to the Khatri-Rao row and the accumulator:
     // there the dot reads the B row through L1 for every nonzero
     constexpr bool BREG = (OP != OP_MTTKRP) && !(sizeof(T) == 8 && (RPL >= 16 || U >= 4));
-    constexpr int BR = BREG ? RPL : 1;
+    // FP64 Phi with up to 8 ranks per lane may take its dot on the FP32 pipe
+    // (df_dot); a B row in registers is then kept as hi/lo floats
+    constexpr bool DFDOT = DF && sizeof(T) == 8 && OP == OP_PHI && RPL <= 8;
+    constexpr bool BREGD = BREG && !DFDOT;  // B row in registers in the working type
+    constexpr int BR = BREGD ? RPL : 1;
+    constexpr int BF = (BREG && DFDOT) ? RPL : 1;
 
     if (la < lb) {
         // does the row at la begin before the run, the row at lb - 1 go on after it?
@@ -793,9 +953,19 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
 #pragma unroll
             for (int r = 0; r < RPL; ++r) acc[h][r] = T(0);
         T brow[BR];  // B row of `brow_row` (loaded once per row, not per nonzero)
+        float bhi[BF], blo[BF];  // or that row cut into hi/lo floats (df_dot)
+        bool bbig = false;       // the cut row has an entry >= 2^31
         int32_t brow_row = cur;
         auto load_brow = [&]() {
-            if constexpr (BREG) load_row<T, BR>(Bm + (int64_t)cur * Rp + col0, brow);
+            if constexpr (BREGD) {
+                load_row<T, BR>(Bm + (int64_t)cur * Rp + col0, brow);
+            } else if constexpr (BREG && DFDOT) {
+                T t[RPL];
+                load_row<T, RPL>(Bm + (int64_t)cur * Rp + col0, t);
+                bbig = false;
+#pragma unroll
+                for (int r = 0; r < RPL; ++r) df_cut((double)t[r], bhi[r], blo[r], bbig);
+            }
         };
         load_brow();
 
@@ -807,7 +977,20 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
             if (!before && !after) {
                 store_row<T, RPL>(out + (int64_t)frow * Rp + col0, v);
                 if (OP == OP_PHI && a.inner) {
-                    if constexpr (BREG) {
+                    if constexpr (BREG && DFDOT) {
+                        // the exact FP64 term only where it could raise the running maximum
+                        // (flushes diverge across a warp's groups, and each FP64 warp
+                        // instruction costs the FP64 pipe the same with two lanes or 32)
+                        if (frow == brow_row && !bbig) {
+                            const float kf = float_below((double)kkt);
+#pragma unroll
+                            for (int r = 0; r < RPL; ++r)
+                                if (kkt_candidate(bhi[r], (double)v[r], kf))
+                                    kkt = tmax(kkt, viol_t(__ldg(Bm + (int64_t)frow * Rp + col0 + r), v[r]));
+                            return;
+                        }
+                    }
+                    if constexpr (BREGD) {
                         if (frow == brow_row) {
 #pragma unroll
                             for (int r = 0; r < RPL; ++r) kkt = tmax(kkt, viol_t(brow[r], v[r]));
@@ -919,17 +1102,66 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
                 for (int u = 0; u < U; ++u) v[u] = xx[u];
             } else {
                 T s[U];
-                if (BREG && fast) {
+                bool fp64dot = true;
+                if constexpr (DFDOT) {
+                    // <B[i_n], pi>, the lanes' sum and x / max(s, eps) on the FP32 pipe,
+                    // unless an operand or x is outside their ranges somewhere in the group
+                    float2 s2[U];
+                    bool big = false;
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
-                        if constexpr (BREG) s[u] = dot_regs<T, RPL>(brow, pi[u]);
-                    }
-                } else {
+                        df_check_x((double)xx[u], big);
+                        // one dot for fast and slow groups alike (converged across the warp)
+                        float bh[RPL], bl[RPL];
+                        if (BREG && fast) {
+                            if constexpr (BREG) {
 #pragma unroll
-                    for (int u = 0; u < U; ++u)
-                        s[u] = dot_global<T, RPL>(Bm + (int64_t)rr[u] * Rp + col0, pi[u]);
+                                for (int r = 0; r < RPL; ++r) {
+                                    bh[r] = bhi[r];
+                                    bl[r] = blo[r];
+                                }
+                            }
+                        } else {
+                            T brw[RPL];
+                            load_row<T, RPL>(Bm + (int64_t)rr[u] * Rp + col0, brw);
+#pragma unroll
+                            for (int r = 0; r < RPL; ++r) df_cut((double)brw[r], bh[r], bl[r], big);
+                        }
+                        s2[u] = df_dot<RPL>(bh, bl, pi[u], big);
+                    }
+                    if constexpr (BREG) big = big || (fast && bbig);
+                    fp64dot = __any_sync(gmask, big);
+                    if (!fp64dot) {
+                        if constexpr (G == 1) {
+#pragma unroll
+                            for (int u = 0; u < U; ++u) v[u] = (T)df_divide((double)xx[u], s2[u], eps_hi, eps_lo);
+                        } else {
+                            const float2 tot = group_reduce_scatter_df<G, U>(s2, lane, gmask);
+                            T xm = xx[0];
+#pragma unroll
+                            for (int u = 1; u < U; ++u)
+                                if (u_mine == u) xm = xx[u];
+                            const T vm = (T)df_divide((double)xm, tot, eps_hi, eps_lo);
+#pragma unroll
+                            for (int u = 0; u < U; ++u) v[u] = __shfl_sync(gmask, vm, gbase + u * LPU);
+                        }
+                    }
                 }
-                if constexpr (G == 1) {
+                if (fp64dot) {
+                    if (BREGD && fast) {
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            if constexpr (BREGD) s[u] = dot_regs<T, RPL>(brow, pi[u]);
+                        }
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            s[u] = dot_global<T, RPL>(Bm + (int64_t)rr[u] * Rp + col0, pi[u]);
+                    }
+                }
+                if (!fp64dot) {
+                    // v done on the FP32 pipe above
+                } else if constexpr (G == 1) {
 #pragma unroll
                     for (int u = 0; u < U; ++u) {
                         if (OP == OP_PHI) {
@@ -981,7 +1213,31 @@ __device__ __forceinline__ bool phi_tile_body(const PhiArgs &a, const int t, uns
                     }
                 }
             }
-            if (fast) {
+            if constexpr (DF && sizeof(T) == 8) {
+                // Row changes (slow batches only) flush the run's sum; the scale-add
+                // itself runs for every group of the warp together, fast or slow, a
+                // nonzero past the run's end adding 0 * pi: each FP64 warp
+                // instruction costs the FP64 pipe the same with two lanes or 32.
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    if (!fast && q + u < lb && rr[u] != cur) {
+                        if (OP != OP_LL) {
+                            flush(cur, first_run, false);
+#pragma unroll
+                            for (int h = 0; h < NACC; ++h)
+#pragma unroll
+                                for (int r = 0; r < RPL; ++r) acc[h][r] = T(0);
+                        }
+                        first_run = false;
+                        cur = rr[u];
+                    }
+                    if (OP != OP_LL) {
+                        const T w = (fast || q + u < lb) ? v[u] : T(0);
+#pragma unroll
+                        for (int r = 0; r < RPL; ++r) acc[u % NACC][r] = fma(w, pi[u][r], acc[u % NACC][r]);
+                    }
+                }
+            } else if (fast) {
                 if (OP != OP_LL) {
 #pragma unroll
                     for (int u = 0; u < U; ++u)
@@ -1054,6 +1310,23 @@ __global__ void __launch_bounds__(THREADS) phi_tile_kernel(const PhiArgs a) {
     __syncthreads();
     uint32_t phase = 0;
     phi_tile_body<T, NM1, RPL, G, OP, THREADS, U, PI>(a, blockIdx.x, smem_raw, red, &bar, phase);
+}
+
+// The FP64 Phi kernel with the divisor on the FP32 pipe.  With four or more
+// lanes per nonzero it runs at five blocks per SM (registers held to 96, a
+// few spilled): measured on GB300 4-6% faster on the 3-way R = 32 and 5-way
+// R = 32 and 64 tensors; with two lanes (R = 16, whose 2048-nonzero stages
+// would then take 213 KB of an SM's shared memory) it was 3-4% slower, so
+// those are held to four blocks (128 registers).
+template <typename T, int NM1, int RPL, int G, int OP, int THREADS, int U, bool PI>
+__global__ void __launch_bounds__(THREADS, G >= 4 ? 5 : 4) phi_tile_kernel_df(const PhiArgs a) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ double red[THREADS / 32];
+    __shared__ __align__(8) uint64_t bar;
+    if (threadIdx.x == 0) stage_barrier_init(&bar);
+    __syncthreads();
+    uint32_t phase = 0;
+    phi_tile_body<T, NM1, RPL, G, OP, THREADS, U, PI, true>(a, blockIdx.x, smem_raw, red, &bar, phase);
 }
 
 // The same with registers held to four resident blocks per SM (64 per

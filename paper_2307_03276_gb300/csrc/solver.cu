@@ -32,7 +32,8 @@ cpapr_status configure_mode(cpapr_ctx *ctx, int n, int lanes, int tile, int redu
 
 static cpapr_status build_inner_graph(cpapr_ctx *ctx, int n, double tol, int max_inner) {
     if (ctx->graph_exec[n]) {
-        if (ctx->graph_max_inner[n] == max_inner && ctx->graph_tol[n] == tol) return CPAPR_OK;
+        if (ctx->graph_max_inner[n] == max_inner && ctx->graph_tol[n] == tol && ctx->graph_route[n] == phi_route(ctx, n))
+            return CPAPR_OK;
         cudaGraphExecDestroy(ctx->graph_exec[n]);
         ctx->graph_exec[n] = nullptr;
     }
@@ -82,6 +83,7 @@ static cpapr_status build_inner_graph(cpapr_ctx *ctx, int n, double tol, int max
     if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGraphInstantiate");
     ctx->graph_exec[n] = exec;
     ctx->graph_max_inner[n] = max_inner;
+    ctx->graph_route[n] = phi_route(ctx, n);
     ctx->graph_tol[n] = tol;
     return CPAPR_OK;
 }
@@ -128,12 +130,17 @@ cpapr_status mu_solve(cpapr_ctx *ctx, double tol, int max_outer, int max_inner, 
     int outer = 0, total_inner = 0;
     bool conv = false;
     double kkt_last = 0.0;
+    const uint32_t all = (1u << N) - 1u;
+    if (max_outer > 0) CPAPR_TRY(ensure_routes(ctx, all));
     for (int k = 0; k < max_outer; ++k) {
         const bool shift = ctx->k_total > 0;
         for (int n = 0; n < N; ++n) CPAPR_TRY(enqueue_mode(ctx, n, tol, max_inner, shift));
+        // the next outer iteration's routes, read back with the inner states
+        if (k + 1 < max_outer) CPAPR_TRY(queue_routes(ctx, all));
         CPAPR_CUDA(ctx, cudaMemcpyAsync(ctx->host->inner, ctx->inner, sizeof(InnerState) * N, cudaMemcpyDeviceToHost,
                                         ctx->stream));
         CPAPR_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+        if (k + 1 < max_outer) take_routes(ctx, all);
         ctx->k_total += 1;
         ++outer;
         bool all_first = true;
@@ -191,6 +198,7 @@ cpapr_status batch_mu_solve(cpapr_ctx *const *ctxs, int count, double tol, int m
             any = true;
             cpapr_ctx *c = ctxs[i];
             const bool shift = c->k_total > 0;
+            CPAPR_TRY(ensure_routes(c, (1u << c->N) - 1u));
             for (int n = 0; n < c->N; ++n) CPAPR_TRY(enqueue_mode(c, n, tol, max_inner, shift));
             CPAPR_CUDA(c, cudaMemcpyAsync(hs[i].data(), c->inner, sizeof(InnerState) * c->N, cudaMemcpyDeviceToHost,
                                           c->stream));
