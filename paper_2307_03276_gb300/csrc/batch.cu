@@ -629,7 +629,8 @@ cpapr_status batch_solve_t(cpapr_ctx *const *ctxs, int count, double tol, int ma
     for (int i = 0; i < count; ++i) {
         CPAPR_CUDA(ctxs[i], cudaStreamSynchronize(ctxs[i]->stream));
         ctxs[i]->pi_mode_built = -1;  // the batched solve changes every factor
-        for (int m = 0; m < N; ++m) factor_changed(ctxs[i], m, kPairStale);
+        if (max_outer > 0)            // and normalises it, as mu_solve does
+            for (int m = 0; m < N; ++m) factor_changed(ctxs[i], m, kPairNormalised);
     }
     // every tensor needs a rank class of the batched kernel and the segmented
     // reduction; it keeps its own tile size (tuned or heuristic) as long as
