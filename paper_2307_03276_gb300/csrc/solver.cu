@@ -300,7 +300,7 @@ static bool choice_fits(const cpapr_ctx *ctx, const TuneChoice &c) {
     return phi_smem_for((int)ctx->esize, ctx->N - 1, c.tile, ctx->Rp, c.lanes) <= kMaxPhiSmem;
 }
 
-// Times each supported (lanes, tile, reduction, Pi form) choice on the
+// Times each supported (lanes, tile, reduction, Pi form) choice that Phi reads on the
 // tensor's own data, one Phi per candidate after a warm-up, and keeps the
 // fastest per mode -- the analogue of the paper's Kokkos policy grid search
 // (league / team / vector sizes, Experiments 3 to 6), chosen per mode
@@ -344,13 +344,21 @@ cpapr_status autotune(cpapr_ctx *ctx) {
         bc.tile = ctx->mode[n].tile_nnz;
         bc.reduction = ctx->mode[n].reduction;
         bc.pi = ctx->mode[n].pi;
-        const int tiles[] = {1024, 2048, 4096, 8192};
+        // below 1024 nonzeros only where larger tiles would leave SMs idle (an inner
+        // iteration of 1e4 nonzeros, R = 10: 25.8 us, 33.8 with the best of the larger)
+        std::vector<int> tiles;
+        if (ceil_div(ctx->nnz, 1024) < 152) tiles = {64, 128, 256, 512};
+        for (int t : {1024, 2048, 4096, 8192}) tiles.push_back(t);
+        // lanes that Phi does not look at keep the heuristic's (or the caller's): timing
+        // them would choose MTTKRP's and the log-likelihood's lanes by noise
+        const int lanes0 = ctx->mode[n].lanes;
         // the materialised Khatri-Rao rows are a candidate where their buffer
         // fits (the fixed cost of building them once per inner loop is not
         // timed: it is spread over the inner iterations)
         const int npi = pi_fits(ctx) ? 2 : 1;
         for (int lanes = 1; lanes <= 32; lanes <<= 1) {
             if (!phi_config_supported((int)ctx->esize, ctx->N - 1, Rp, lanes)) continue;
+            if (ctx->esize == 4 && lanes != lanes0) continue;
             for (int tile : tiles) {
                 // MTTKRP and the log-likelihood share the mode's tiles and stage every
                 // coordinate stream: keep room for two of their blocks per SM
@@ -359,6 +367,7 @@ cpapr_status autotune(cpapr_ctx *ctx) {
                     const int red = cand % 2 ? CPAPR_REDUCE_SEGMENTED : CPAPR_REDUCE_ATOMIC;
                     const int pi = cand / 2;
                     CPAPR_TRY(configure_mode(ctx, n, lanes, tile, red));
+                    if (uses_pairs(ctx, n) && lanes != lanes0 && Rp / lanes0 <= 8) continue;
                     CPAPR_TRY(configure_pi(ctx, n, pi));
                     CPAPR_TRY(prepare_phi(ctx, n));
                     // a fresh inner state: not done, violation slots clear
