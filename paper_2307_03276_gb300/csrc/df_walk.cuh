@@ -34,8 +34,12 @@
 // (u^2 each), and the FP32 sums of the two-sum errors, FMA errors and cross
 // terms, each at most u of its product and rounded to u of itself: k^2 u^2 + 4 k u^2
 // < 40 u^2 at worst and a few u^2 in the mean; the quotient's remainder is exact to
-// 2 u^2.  That is below 3e-13 at worst; the mean over Phi entries is measured
-// smaller than with the FP64 scale-add and the one-step quotient it replaces.
+// 2 u^2.  That is below 3e-13 at worst.  The scale-add of n terms rounds C, at most (2 + n) u
+// of the sum, three times a term: (3 n (2 + n) + n) u^2, 3e-12 for the 16 terms between two
+// moves to FP64 if every rounding had one sign, some 1e-15 as they come.  Phi entries
+// of the timed workloads are within 1e-14 to 3e-14 of 64-bit results, like those of
+// the FP64 scale-add and the one-step quotient before (a few parts larger on the 4-way
+// solve, smaller on others).
 #pragma once
 
 #include "direct.cuh"
@@ -66,9 +70,10 @@ __device__ __forceinline__ void df_cut(double x, int s, float &hi, float &lo) {
     const bool keep = e >= 1023 - 126;
     // the first 23 fraction bits with the exponent rebased from 1023 to 127
     const float h = __uint_as_float(__funnelshift_l(L, H, 3) + ((uint32_t)(s - 896) << 23));
-    // the next 29 fraction bits (24 kept) times 2^(e - 1075), in two exact steps
+    // the next 29 fraction bits (24 kept) times 2^(e - 1075), in two exact steps that
+    // stay in the float range for every e kept
     const float m = __uint2float_rz(L & 0x1fffffffu);
-    const float l = __fmul_rn(m * __uint_as_float((uint32_t)(e - 1075 + 64 + 127) << 23), 0x1p-64f);
+    const float l = __fmul_rn(m * __uint_as_float((uint32_t)(e - 1023 + 127) << 23), 0x1p-52f);
     const float t = h + l;
     hi = keep ? t : 0.f;
     lo = keep ? l - (t - h) : 0.f;
