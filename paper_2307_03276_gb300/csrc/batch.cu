@@ -170,6 +170,7 @@ __global__ void __launch_bounds__(batch_block<T, OP>(), batch_min_blocks<T, OP>(
         if (it >= nitems) break;
         const int2 w = items[it];
         if constexpr (OP == OP_PHI) {
+            if (desc[w.x].a.inner->done) continue;
             // the tile reads its arguments from shared memory (the previous
             // item's last reads are behind the barriers above)
             __shared__ PhiArgs s_a;
@@ -177,7 +178,6 @@ __global__ void __launch_bounds__(batch_block<T, OP>(), batch_min_blocks<T, OP>(
             for (int k = threadIdx.x; k < (int)(sizeof(PhiArgs) / 4); k += batch_block<T, OP>())
                 reinterpret_cast<uint32_t *>(&s_a)[k] = reinterpret_cast<const uint32_t *>(&desc[w.x].a)[k];
             __syncthreads();
-            if (s_a.inner->done) continue;
             const int cfg = desc[w.x].cfg;
             if constexpr (sizeof(T) == 8) {
                 if (s_a.pi) {
