@@ -287,15 +287,39 @@ static void heuristic_config(const cpapr_ctx *ctx, int pi, ModeLayout &L, int *l
     // FP32: at most one tile per SM below 1024 nonzeros, one and a half where eight or
     // more lanes per nonzero make long runs (1e4 nonzeros, R = 16: 34 -> 15 us; 1e5: 32 ->
     // 24; R = 32: 39 -> 28); 2048 only from 4 tiles per SM on, or 8.  The batched solver
-    // takes the same tiles, so that a tensor's FP32 sums keep one order in both,
-    // and larger numbers of them cost it more than a lone launch gains (64 tensors:
-    // 27.5 ms at one tile per SM, 34 at four).
+    // takes these too: larger numbers of them cost it more than a lone launch gains (64
+    // tensors: 27.5 ms at one tile per SM, 34 at four).
     const bool wide = g >= 8;
     while (!f64 && *tile > 1024 && ceil_div(ctx->nnz, *tile / 2) < (wide ? 2 : 1) * kSmallTiles) *tile /= 2;
     const int few = f64 ? kSmallTiles : wide ? kSmallTiles * 3 / 8 : kSmallTiles / 4;
     while (*tile > 64 && ceil_div(ctx->nnz, *tile / 2) < few) {
         *tile /= 2;
         L.batch_sh += f64 ? 1 : 0;
+    }
+    // The direct Phi launches of a lone FP32 tensor run 8 blocks of 128 threads per SM:
+    // above the sizes where the tiles so far are small ones, theirs are the smallest
+    // that all run at once.  A few tiles more than one wave doubled a launch's time, and
+    // half a wave of larger ones left the memory idle (4-way, materialised, us at 512 /
+    // 1024 / 2048 / 4096 / 8192 nonzeros per tile: 4e5, R = 32, 24 / 32 / 46 / 75 / 134; 7e5, R = 16,
+    // 30 / 26 / 33 / 48 / 77; 2e6 52 / 42 / 35 / 47 / 73; 5e6, R = 8, 111 / 80 / 70 / 67 / 58; 8e6, R = 16, 157 /
+    // 128 / 119 / 106 / 98).  Rows formed in place gain from 8192 in a 3-way tensor up to
+    // rank 16 only (5e6, us at 2048 / 8192: R = 16, 87 / 85; R = 32, 122 / 136; 5-way, R = 16,
+    // 150 / 157).  The batched solver keeps the tiles above (with these 22.0 -> 22.7 ms
+    // on 64 tensors), so that an FP32 tensor's sums take another order there.
+    if (!f64) {
+        const bool wide_rank = ctx->Rp >= 64;
+        int direct = *tile;
+        if (wide_rank || *tile >= 1024) {
+            int t = wide_rank ? 64 : 256;
+            const int most = pi || (ctx->N <= 3 && ctx->Rp <= 16) ? 8192 : 4096;
+            while (t < most && ceil_div(ctx->nnz, t) > kDirectWave) t *= 2;
+            if (ceil_div(ctx->nnz, t) <= kDirectWave) direct = t;
+        }
+        const int staged = *tile;
+        *tile = std::min(direct, staged);
+        while ((*tile << L.sh) < staged) ++L.sh;
+        while ((*tile << L.sh_df) < direct) ++L.sh_df;
+        L.batch_sh = L.sh;
     }
     *reduction = CPAPR_REDUCE_SEGMENTED;
 }

@@ -75,8 +75,8 @@ struct ModeLayout {
     int32_t *split = nullptr;      // [3 * nsplit] (row, first tile, last tile)
     int32_t *tsplit = nullptr;     // [ntiles] split of each tile's head partial, or -1
     int32_t *splitcnt = nullptr;   // [nsplit] partial counters of the tile kernel (zero between launches)
-    // a launch takes 2^k of these tiles as one (heuristic_config): k = sh, sh_df for
-    // the kernels over float pairs, batch_sh in the batched solver
+    // a launch takes 2^k of these tiles as one (heuristic_config): k = sh, sh_df for Phi
+    // over float pairs and the direct FP32 Phi, batch_sh in the batched solver
     int32_t sh = 0, sh_df = 0, batch_sh = 0;
     bool late = false;             // the float pairs are slower than the FP64 rows by now (route.cu)
     int32_t pi = 0;                // 1: Phi streams the materialised Khatri-Rao rows (built per outer iteration)
@@ -175,6 +175,8 @@ constexpr int kSmallTiles = 152 * 4;
 constexpr int kDfTile = 512;
 constexpr int kDfRun = 128;
 constexpr int kDfLaunchTiles = 152 * 9;
+// blocks of a direct FP32 launch (direct.cuh) that run at once
+constexpr int kDirectWave = 152 * 8;
 
 // ---- error plumbing ------------------------------------------------------
 cpapr_status fail(cpapr_ctx *ctx, cpapr_status st, const std::string &msg);
@@ -248,7 +250,7 @@ void take_routes(cpapr_ctx *ctx, uint32_t modes);
 cpapr_status ensure_routes(cpapr_ctx *ctx, uint32_t modes);
 // log2 of the table tiles per tile of mode n's Phi launch
 inline int phi_shift(const cpapr_ctx *ctx, int n) {
-    return uses_pairs(ctx, n) ? ctx->mode[n].sh_df : ctx->mode[n].sh;
+    return ctx->esize == 4 || uses_pairs(ctx, n) ? ctx->mode[n].sh_df : ctx->mode[n].sh;
 }
 cpapr_status ensure_pair_storage(cpapr_ctx *ctx);
 cpapr_status launch_factor_pairs(cpapr_ctx *ctx, int m, bool from_data);
