@@ -59,9 +59,9 @@ __device__ __forceinline__ float direct_divide(float x, float s, float eps) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(m));
     const float q = x * r;
     const float c = fmaf(fmaf(-q, m, x), r, q);
-    // (huge and tiny divisors, whose reciprocal leaves the float range, and
-    // quotients beyond it, whose correction would be NaN)
-    return m > 0x1p-100f && m < 0x1p100f && q < __int_as_float(0x7f800000) ? c : __fdiv_rn(x, m);
+    // (huge divisors, whose reciprocal is 0; tiny ones and quotients beyond the float
+    // range, whose correction is NaN)
+    return m < 0x1p100f && q < __int_as_float(0x7f800000) ? c : __fdiv_rn(x, m);
 }
 
 // shared memory of a tile: partial-row slots, their rows, the rows finished here
@@ -128,8 +128,9 @@ __device__ __forceinline__ void direct_tile(const PhiArgs &a, const int t, unsig
         for (int r = 0; r < 4; ++r) {
             const float y = (acc[0][r] + acc[1][r]) - kc[r];
             const float s = ks[r] + y;
-            // (a sum that overflows stays infinite: its correction would be NaN)
-            kc[r] = s < __int_as_float(0x7f800000) ? (s - ks[r]) - y : 0.f;
+            // (finite even where the sum is not, so that it stays infinite: its correction
+            // would be infinite or NaN, and fminf returns the other operand of a NaN)
+            kc[r] = fminf((s - ks[r]) - y, 0x1.fffffep127f);
             ks[r] = s;
             acc[0][r] = acc[1][r] = 0.f;
         }
