@@ -622,6 +622,7 @@ cpapr_status cpapr_create(int32_t nmodes, const int64_t *dims, int64_t nnz, cons
             ctx->mode[n].sh_df = h.sh_df;
             ctx->mode[n].batch_sh = h.batch_sh;
         }
+        ctx->mode[n].batch_tile = ctx->mode[n].tile_nnz << ctx->mode[n].batch_sh;
         CR_TRY(configure_pi(ctx, n, pi));
     }
     // after everything the context cannot do without

@@ -78,6 +78,7 @@ struct ModeLayout {
     // a launch takes 2^k of these tiles as one (heuristic_config): k = sh, sh_df for Phi
     // over float pairs and the direct FP32 Phi, batch_sh in the batched solver
     int32_t sh = 0, sh_df = 0, batch_sh = 0;
+    int32_t batch_tile = 0;        // the built-in choice for the batched solver, before any tuning
     bool late = false;             // the float pairs are slower than the FP64 rows by now (route.cu)
     int32_t pi = 0;                // 1: Phi streams the materialised Khatri-Rao rows (built per outer iteration)
     int32_t nempty = 0;

@@ -126,11 +126,12 @@ __global__ void __launch_bounds__(32 * kProbeWarps) route_probe_kernel(const __g
 
 // Share of nonzeros summed again up to which the pairs are not slower, as measured
 // over 36 outer iterations (ms an outer iteration with all modes on pairs against
-// all on FP64 rows, and the share of the mode that has most).  3-way 1e7, R = 32, materialised: 31.4
-// against 33.2 at 0.0009, 33.1 at 0.0027, 41 at 0.012 (so it leaves them by the 23rd).  3-way 3e6, R = 64: 15.4 against 19.2 at
-// 0.0022, 20.5 at 0.0061.  3-way 1.3e6, R = 16: 4.4 against 4.9 at 0.006.  4-way 1.5e6, R = 100:
-// 25.4 against 56 at 0.07.  6-way 2e6, R = 40: 29.9 against 32.4 at 0.01.  In place they hold
-// longer: 3-way 1e7 41 against 44 at 0.012.
+// all on FP64 rows, and the share of the mode that has most).  3-way 1e7, R = 32,
+// materialised: 31.4 against 33.2 at 0.0009, 33.1 at 0.0027, 41 at 0.012 (so it leaves them
+// by the 23rd).  3-way 3e6, R = 64: 15.4 against 19.2 at 0.0022, 20.5 at 0.0061.  3-way 1.3e6,
+// R = 16: 4.4 against 4.9 at 0.006.  4-way 1.5e6, R = 100: 56 against 25.4 at 0.07.  6-way 2e6,
+// R = 40: 29.9 against 32.4 at 0.01.  In place they hold longer: 3-way 1e7 41 against 44 at
+// 0.012.
 constexpr double kResumLimit = 0.0015;
 
 }  // namespace

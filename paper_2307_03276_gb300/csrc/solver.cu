@@ -261,6 +261,16 @@ static std::string tune_key(const cpapr_ctx *ctx, int n) {
     return buf;
 }
 
+// A tuned choice for mode n.  The batched solver takes its tiles together up to the
+// built-in size: tuned alone, a small tensor has smaller ones than the batch wants
+// (64 tensors, FP32: 11.6 ms a step with them, 8.8 with 1024 nonzeros at least, 8.1 untuned).
+static cpapr_status configure_tuned(cpapr_ctx *ctx, int n, int lanes, int tile, int reduction, int pi) {
+    CPAPR_TRY(configure_mode(ctx, n, lanes, tile, reduction));
+    ModeLayout &L = ctx->mode[n];
+    while ((L.tile_nnz << (L.batch_sh + 1)) <= L.batch_tile) ++L.batch_sh;
+    return configure_pi(ctx, n, pi);
+}
+
 static std::mutex g_tune_mu;
 
 static bool tune_lookup(const char *path, const std::string &key, TuneChoice *out) {
@@ -319,8 +329,7 @@ cpapr_status autotune(cpapr_ctx *ctx) {
         keys[n] = tune_key(ctx, n);
         TuneChoice c;
         if (cache && tune_lookup(cache, keys[n], &c) && choice_fits(ctx, c)) {
-            CPAPR_TRY(configure_mode(ctx, n, c.lanes, c.tile, c.reduction));
-            CPAPR_TRY(configure_pi(ctx, n, c.pi));
+            CPAPR_TRY(configure_tuned(ctx, n, c.lanes, c.tile, c.reduction, c.pi));
         } else if (ctx->opt.autotune) {
             todo.push_back(n);
         }
@@ -389,8 +398,7 @@ cpapr_status autotune(cpapr_ctx *ctx) {
                 }
             }
         }
-        CPAPR_TRY(configure_mode(ctx, n, bc.lanes, bc.tile, bc.reduction));
-        CPAPR_TRY(configure_pi(ctx, n, bc.pi));
+        CPAPR_TRY(configure_tuned(ctx, n, bc.lanes, bc.tile, bc.reduction, bc.pi));
         CPAPR_CUDA(ctx, cudaMemsetAsync(inner, 0, sizeof(InnerState), ctx->stream));
         if (cache) tune_store(cache, keys[n], bc, best / 3.f);
     }
