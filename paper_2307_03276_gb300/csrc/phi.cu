@@ -22,6 +22,10 @@ cudaError_t launch_phi_df_n2(const PhiArgs &, cudaStream_t, const cudaAccessPoli
 cudaError_t launch_phi_df_n3(const PhiArgs &, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_phi_df_n4(const PhiArgs &, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_phi_df_pi(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_phi_pipe_n0(const PhiArgs &, int, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_phi_pipe_n2(const PhiArgs &, int, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_phi_pipe_n3(const PhiArgs &, int, int, cudaStream_t, const cudaAccessPolicyWindow *);
+cudaError_t launch_phi_pipe_n4(const PhiArgs &, int, int, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_direct_f32_n0(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_direct_f32_n2(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
 cudaError_t launch_direct_f32_n3(const PhiArgs &, int, cudaStream_t, const cudaAccessPolicyWindow *);
@@ -64,6 +68,14 @@ static cudaError_t dispatch(const cpapr_ctx *ctx, const PhiArgs &a, int rpl, int
             case 3: return launch_phi_df_n3(a, ctx->stream, win);
             case 4: return launch_phi_df_n4(a, ctx->stream, win);
             default: return launch_phi_df_n0(a, ctx->stream, win);
+        }
+    }
+    if (a.route == kRoutePipe && op == OP_PHI) {
+        switch (nm1) {
+            case 2: return launch_phi_pipe_n2(a, rpl, lanes, ctx->stream, win);
+            case 3: return launch_phi_pipe_n3(a, rpl, lanes, ctx->stream, win);
+            case 4: return launch_phi_pipe_n4(a, rpl, lanes, ctx->stream, win);
+            default: return launch_phi_pipe_n0(a, rpl, lanes, ctx->stream, win);
         }
     }
     if (ctx->esize == 4 && op != OP_LL && !(op == OP_MTTKRP && nm1 == 2)) {
