@@ -591,7 +591,8 @@ def ncu_traffic(T, dtype, mat, info, inner_per_mode):
 def on_pairs(T, info) -> bool:
     """Whether the FP64 Phi launches run on float pairs (the library's automatic
     choice): 8 or fewer ranks per lane and at least 608 tiles of 2048 nonzeros
-    (1024 from rank 17 on)."""
+    (1024 from rank 17 on), and a model not so late in a solve that its modes have
+    gone back to FP64 rows (the default workloads' have not within 20 steps)."""
     rp = info.rank_padded
     tile = 2048 if rp <= 16 else 1024
     return rp // max(int(info.rank_lanes[0]), 1) <= 8 and -(-T.nnz // tile) >= 608
